@@ -24,6 +24,14 @@
 // the survivors of one buffer into the other (warp ballots, one atomic per
 // warp) and appends the new entrance particles.  Counts live on the device,
 // so steps need no host synchronisation.
+//
+// What bounds a step is the FP64 pipe (two lanes per clock and SM here, a
+// 64th of the float rate), not memory (0.5% of HBM).  So decisions are taken
+// in float or integers wherever those can be certain of the double's answer
+// (which fibers are near, which direction candidates lie in the disc, the
+// wall and edge tests), the double test runs only in between, and the
+// direction's square root and divisions share their Newton steps.  The
+// results are the same bits.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -72,17 +80,25 @@ struct Fiber {
   int pad;
 };
 
+// the same for the float test of which fibers are near: centre, and a bound
+// that the float distance squared exceeds only where the double distance is
+// beyond both the reflecting radius and the shell
+struct Near {
+  float cx, cy, d2, pad;
+};
+
 struct Args {
   int nx, ny, nx_pad, nfib;
   int nspecies;
   int periodic;      // box periodic in x and y: no inlet, outlet or walls
   int homogeneous;   // every particle reacts, wherever it is
-  int pad;
+  int plain;         // step length outside unit_step's range
   double dt, len, delta;   // time step, diffusion step length, shell width
   double hk1, hk2;         // homogeneous rates (A -> B, B -> C)
   unsigned long long seed;
   const double *u;         // [2][ny][nx_pad]
   const Fiber *fib;
+  const Near *near;
 };
 
 struct Buf {
@@ -91,25 +107,50 @@ struct Buf {
   int *s;
 };
 
-// Counters (device, unsigned long long): the particle count of each buffer,
-// the outflow of each species since the last reset, the overflow flag.  A
-// buffer's count can pass the capacity when particles are dropped for lack
+// Counters (device, unsigned long long): three particle counts in turn (of
+// the buffer read, of the buffer written, and one that the step clears for
+// the next), the outflow of each species since the last reset, the overflow
+// flag.  A count can pass the capacity when particles are dropped for lack
 // of room (the appends count them, the slots refuse them), so every reader
 // takes min(count, capacity).
-enum { kCount0 = 0, kCount1 = 1, kOut = 2, kOverflow = 5, kCounters = 8 };
+enum { kCount = 0, kOut = 3, kOverflow = 6, kCounters = 8 };
 
 __device__ inline double dadd(double a, double b) { return __dadd_rn(a, b); }
 __device__ inline double dsub(double a, double b) { return __dsub_rn(a, b); }
 __device__ inline double dmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ inline double ddiv(double a, double b) { return __ddiv_rn(a, b); }
 
+__device__ inline long long bits(double v) { return __double_as_longlong(v); }
+// v < t, for a threshold t that is not zero, by integer comparison of the
+// bit patterns (a comparison in double is an FP64 operation); a NaN that
+// arithmetic made is greater than every number
+__device__ inline bool below(double v, double t) {
+  const long long a = bits(v), b = bits(t);
+  return (a ^ ((a >> 63) & 0x7FFFFFFFFFFFFFFFll)) <
+         (b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFll));
+}
+
+// floor(v) as a double and as an integer.  Adding 1.5 * 2^52 rounded down
+// leaves floor(v) in the low bits of the sum, for |v| < 2^30.
+__device__ inline double floor_int(double v, int &i) {
+  constexpr double kMagic = 6755399441055744.0;
+  if ((__double2hiint(v) & 0x7FFFFFFF) < 0x41D00000) {
+    const double m = __dadd_rd(v, kMagic);
+    i = __double2loint(m);
+    return dsub(m, kMagic);
+  }
+  const double f = floor(v);
+  i = static_cast<int>(f);
+  return f;
+}
+
 // u at (px, py): bilinear in the four nodes around the point (node indices
 // clamped to the lattice)
 __device__ inline void velocity(const Args &a, double px, double py,
                                 double &ux, double &uy) {
-  const double fx0 = floor(px), fy0 = floor(py);
+  int i0, j0;
+  const double fx0 = floor_int(px, i0), fy0 = floor_int(py, j0);
   const double fx = dsub(px, fx0), fy = dsub(py, fy0);
-  int i0 = static_cast<int>(fx0), j0 = static_cast<int>(fy0);
   int i1 = i0 + 1, j1 = j0 + 1;
   i0 = min(max(i0, 0), a.nx - 1);
   i1 = min(max(i1, 0), a.nx - 1);
@@ -127,6 +168,68 @@ __device__ inline void velocity(const Args &a, double px, double py,
                  dmul(w01, a.u[n01])), dmul(w11, a.u[n11]));
   uy = dadd(dadd(dadd(dmul(w00, a.u[plane + n00]), dmul(w10, a.u[plane + n10])),
                  dmul(w01, a.u[plane + n01])), dmul(w11, a.u[plane + n11]));
+}
+
+// 2 d - 1 of the draw d = k 2^-53 in [0, 1) whose generator output is z
+// (k its top 53 bits): the low 52 bits of k are the mantissa of a number in
+// [1, 2), which is exactly 1 or 2 above the result.
+__device__ inline double centred(unsigned long long z) {
+  const double m = __longlong_as_double(static_cast<long long>(
+      ((z >> 11) & 0xFFFFFFFFFFFFFull) | 0x3FF0000000000000ull));
+  return dsub(m, (z >> 63) ? 1.0 : 2.0);
+}
+// the same to within 2^-23, in float
+__device__ inline float centred_float(unsigned long long z) {
+  return static_cast<float>(static_cast<int>(
+             static_cast<unsigned>(z >> 32) ^ 0x80000000u)) * 0x1.0p-31f;
+}
+
+// (len v1 / r, len v2 / r), r = sqrt(q), each operation correctly rounded.
+// The square root is Goldschmidt's iteration from a float estimate with
+// Markstein's final correction, the quotients Markstein's division by a
+// shared reciprocal (P. Markstein, "Computation of elementary functions on
+// the IBM RISC System/6000 processor", 1990): the reciprocal is correctly
+// rounded except for an all-ones mantissa, which is divided plainly, and
+// each quotient is corrected twice, the second time from an estimate within
+// an ulp, whose remainder is exact.  24 double operations in place of the
+// roughly 60 of one square root and two divisions.
+__device__ inline void unit_step(const Args &a, double v1, double v2, double q,
+                                 double &sx, double &sy) {
+  const double n1 = dmul(a.len, v1), n2 = dmul(a.len, v2);
+  if (a.plain) {   // a step length whose remainders could leave the range
+    const double r = __dsqrt_rn(q);
+    sx = ddiv(n1, r);
+    sy = ddiv(n2, r);
+    return;
+  }
+  const double y0 = double(rsqrtf(__double2float_rn(q)));
+  double g = q * y0, h = 0.5 * y0;
+  double e = fma(-g, h, 0.5);
+  g = fma(g, e, g);
+  h = fma(h, e, h);
+  e = fma(-g, h, 0.5);
+  g = fma(g, e, g);
+  h = fma(h, e, h);
+  const double r = fma(fma(-g, g, q), h, g);
+  if ((bits(r) & 0xFFFFFFFFFFFFFll) == 0xFFFFFFFFFFFFFll) {
+    sx = ddiv(n1, r);
+    sy = ddiv(n2, r);
+    return;
+  }
+  double y = h + h;
+  y = fma(y, fma(-r, y, 1.0), y);
+  y = fma(y, fma(-r, y, 1.0), y);
+  double s1 = n1 * y, s2 = n2 * y;
+  s1 = fma(fma(-s1, r, n1), y, s1);
+  s2 = fma(fma(-s2, r, n2), y, s2);
+  sx = fma(fma(-s1, r, n1), y, s1);
+  sy = fma(fma(-s2, r, n2), y, s2);
+}
+
+// Whether fiber k may hold (fx, fy) within its reflecting radius or shell.
+__device__ inline bool may_hold(const Near &f, float fx, float fy) {
+  const float dx = fx - f.cx, dy = fy - f.cy;
+  return !(dx * dx + dy * dy > f.d2);
 }
 
 // Mirror p at the circle of radius rp about c if p is inside it:
@@ -156,11 +259,13 @@ __device__ inline double wrap(double v, double lo, double span) {
 
 // The rate that applies to a particle of species s at (px, py), or 0: the
 // first fiber (list order) whose shell rp <= d < rp + delta holds the point
-// and whose catalyst acts on s.
+// and whose catalyst acts on s.  first: the first fiber that may hold it.
 __device__ inline double shell_rate(const Args &a, int s, double px,
-                                    double py) {
+                                    double py, int first) {
   if (a.homogeneous) return s == 0 ? a.hk1 : (s == 1 ? a.hk2 : 0.0);
-  for (int j = 0; j < a.nfib; ++j) {
+  const float fx = __double2float_rn(px), fy = __double2float_rn(py);
+  for (int j = first; j < a.nfib; ++j) {
+    if (!may_hold(a.near[j], fx, fy)) continue;
     const Fiber &f = a.fib[j];
     const double dx = dsub(px, f.cx), dy = dsub(py, f.cy);
     const double d2 = dadd(dmul(dx, dx), dmul(dy, dy));
@@ -198,14 +303,67 @@ __device__ inline long long warp_slot(bool keep, unsigned long long *cnt,
   return slot;
 }
 
-// One time step of every particle of `in` (count in cnt[kin]); survivors go
-// to `out` (count in cnt[kout], zero on entry).
+// New particles of species A with ids id0 .. id0 + m - 1, uniform in the
+// rectangle [x0, x0 + wx) x [-1/2, ny - 1/2), those inside a fiber dropped,
+// appended to `out` by blocks block, block + blocks, ...
+__device__ inline void spawn(const Args &a, const Buf &out,
+                             unsigned long long *cnt, int kout, long long cap,
+                             long long t, unsigned long long id0, long long m,
+                             double x0, double wx, int block, int blocks) {
+  const long long stride = static_cast<long long>(blocks) * kThreads;
+  for (long long base = static_cast<long long>(block) * kThreads; base < m;
+       base += stride) {
+    const long long j = base + threadIdx.x;
+    bool keep = j < m;
+    double px = 0.0, py = 0.0;
+    const unsigned long long id = id0 + static_cast<unsigned long long>(j);
+    if (keep) {
+      const unsigned long long ps = particle_seed(a.seed, id);
+      px = dadd(x0, dmul(wx, draw(ps, t, kSpawnDraw)));
+      py = dadd(-0.5, dmul(static_cast<double>(a.ny), draw(ps, t, kSpawnDraw + 1)));
+      const float fx = __double2float_rn(px), fy = __double2float_rn(py);
+      for (int k = 0; k < a.nfib && keep; ++k) {
+        if (!may_hold(a.near[k], fx, fy)) continue;
+        const Fiber &f = a.fib[k];
+        const double dx = dsub(px, f.cx), dy = dsub(py, f.cy);
+        if (dadd(dmul(dx, dx), dmul(dy, dy)) < dmul(f.rp, f.rp)) keep = false;
+      }
+    }
+    const long long slot = warp_slot(keep, cnt + kout, cap, cnt + kOverflow);
+    if (slot >= 0) {
+      out.x[slot] = px;
+      out.y[slot] = py;
+      out.s[slot] = 0;
+      out.id[slot] = id;
+    }
+  }
+}
+
+// The initial fill.
+__global__ void __launch_bounds__(kThreads)
+    rwpt_spawn_kernel(const Args a, Buf out, unsigned long long *cnt, int kout,
+                      long long cap, long long t, unsigned long long id0,
+                      long long m, double x0, double wx) {
+  spawn(a, out, cnt, kout, cap, t, id0, m, x0, wx, blockIdx.x, gridDim.x);
+}
+
+// One time step: the blocks below `movers` move every particle of `in`
+// (count in cnt[kin]) and append the survivors to `out` (count in cnt[kout],
+// zero on entry), the others append the m new entrance particles; the third
+// count, cnt[kclr], is cleared for the next step.
 __global__ void __launch_bounds__(kThreads)
     rwpt_step_kernel(const Args a, Buf in, Buf out, unsigned long long *cnt,
-                     int kin, int kout, long long cap, long long t) {
+                     int kin, int kout, int kclr, long long cap, long long t,
+                     unsigned long long id0, long long m, int movers) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) cnt[kclr] = 0ull;
+  if (static_cast<int>(blockIdx.x) >= movers) {
+    spawn(a, out, cnt, kout, cap, t, id0, m, -0.5, 1.0, blockIdx.x - movers,
+          gridDim.x - movers);
+    return;
+  }
   const long long n = min(static_cast<long long>(cnt[kin]), cap);
-  const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
-  for (long long base = static_cast<long long>(blockIdx.x) * blockDim.x; base < n;
+  const long long stride = static_cast<long long>(movers) * kThreads;
+  for (long long base = static_cast<long long>(blockIdx.x) * kThreads; base < n;
        base += stride) {
     const long long i = base + threadIdx.x;
     bool keep = i < n;
@@ -226,109 +384,98 @@ __global__ void __launch_bounds__(kThreads)
         px = dadd(px, dmul(a.dt, ux));
         py = dadd(py, dmul(a.dt, uy));
       }
-      // diffusion: a step of length sqrt(4 D dt) in a uniform direction
+      // diffusion: a step of length sqrt(4 D dt) in a uniform direction, the
+      // first candidate of the square inside the unit disc.  The float
+      // squared radius is within 1e-6 of the double's, so only a candidate
+      // near the rim or the centre needs the double.
       if (a.len > 0.0) {
-        double v1 = 1.0, v2 = 0.0, q = 1.0;
-        for (int k = 0; k < kTries; ++k) {
-          const double c1 = dsub(dmul(2.0, draw(ps, t, 2 * k)), 1.0);
-          const double c2 = dsub(dmul(2.0, draw(ps, t, 2 * k + 1)), 1.0);
-          const double q2 = dadd(dmul(c1, c1), dmul(c2, c2));
-          if (q2 > 0.0 && q2 <= 1.0) {
-            v1 = c1;
-            v2 = c2;
-            q = q2;
-            break;
+        const unsigned long long c0 =
+            ps + (static_cast<unsigned long long>(t) * kDraws + 1ull) * kGamma;
+        unsigned long long z1 = 0, z2 = 0;
+        bool found = false;
+        for (int k = 0; k < kTries && !found; ++k) {
+          z1 = mix64(c0 + static_cast<unsigned long long>(2 * k) * kGamma);
+          z2 = mix64(c0 + static_cast<unsigned long long>(2 * k + 1) * kGamma);
+          const float f1 = centred_float(z1), f2 = centred_float(z2);
+          const float q = f1 * f1 + f2 * f2;
+          if (q > 1.00001f) continue;
+          found = true;
+          if (!(q < 0.99999f && q > 1e-5f)) {
+            const double c1 = centred(z1), c2 = centred(z2);
+            const double q2 = dadd(dmul(c1, c1), dmul(c2, c2));
+            found = q2 > 0.0 && q2 <= 1.0;
           }
         }
-        const double r = __dsqrt_rn(q);
-        px = dadd(px, ddiv(dmul(a.len, v1), r));
-        py = dadd(py, ddiv(dmul(a.len, v2), r));
+        const double v1 = found ? centred(z1) : 1.0, v2 = found ? centred(z2) : 0.0;
+        const double q = dadd(dmul(v1, v1), dmul(v2, v2));
+        double sx, sy;
+        unit_step(a, v1, v2, q, sx, sy);
+        px = dadd(px, sx);
+        py = dadd(py, sy);
       }
       // elastic reflections: walls y = -1/2, ny - 1/2 and the fibers
       const double ytop = dsub(static_cast<double>(a.ny), 0.5);
+      int first = a.nfib;   // the first fiber that may hold the particle
       for (int pass = 0; pass < kReflections; ++pass) {
         bool hit = false;
         if (a.periodic) {
           px = wrap(px, -0.5, static_cast<double>(a.nx));
           py = wrap(py, -0.5, static_cast<double>(a.ny));
         } else {
-          if (py < -0.5) {
+          if (below(py, -0.5)) {
             py = dsub(-1.0, py);
             hit = true;
-          } else if (py > ytop) {
+          } else if (below(ytop, py)) {
             py = dsub(dmul(2.0, ytop), py);
             hit = true;
           }
         }
-        for (int k = 0; k < a.nfib; ++k) hit = reflect_fiber(a.fib[k], px, py) || hit;
+        float fx = __double2float_rn(px), fy = __double2float_rn(py);
+        first = a.nfib;
+        for (int k = 0; k < a.nfib; ++k) {
+          if (!may_hold(a.near[k], fx, fy)) continue;
+          first = min(first, k);
+          if (reflect_fiber(a.fib[k], px, py)) {
+            hit = true;
+            fx = __double2float_rn(px);
+            fy = __double2float_rn(py);
+          }
+        }
         if (!hit) break;
+        first = 0;   // moved: any fiber may hold it now
       }
       // reaction with probability k dt
       if (s < a.nspecies - 1) {
-        const double k = shell_rate(a, s, px, py);
+        const double k = shell_rate(a, s, px, py, first);
         if (k > 0.0 && draw(ps, t, kReactDraw) < dmul(k, a.dt)) s += 1;
       }
       // inlet and outlet
       if (!a.periodic) {
         const double xout = dsub(static_cast<double>(a.nx), 0.5);
-        if (!(px < xout)) {
+        if (!below(px, xout)) {
           outflow = s;
           keep = false;
-        } else if (px < -0.5) {
+        } else if (below(px, -0.5)) {
           if (s == 0)
             keep = false;          // back into the reservoir of A
           else
             px = dsub(-1.0, px);   // B and C: the entrance reflects
         }
-        if (keep && s == 0 && px < 0.5) keep = false;  // strip: re-seeded
+        if (keep && s == 0 && below(px, 0.5)) keep = false;  // strip: re-seeded
       }
     }
     // outflow counts (one atomic per warp and species)
 #pragma unroll
     for (int sp = 0; sp < 3; ++sp) {
-      const unsigned m = __ballot_sync(0xffffffffu, outflow == sp);
-      if (m && (threadIdx.x & 31) == __ffs(m) - 1)
-        atomicAdd(cnt + kOut + sp, static_cast<unsigned long long>(__popc(m)));
+      const unsigned mask = __ballot_sync(0xffffffffu, outflow == sp);
+      if (mask && (threadIdx.x & 31) == __ffs(mask) - 1)
+        atomicAdd(cnt + kOut + sp, static_cast<unsigned long long>(__popc(mask)));
     }
     const long long slot = warp_slot(keep, cnt + kout, cap, cnt + kOverflow);
     if (slot >= 0) {
       out.x[slot] = px;
       out.y[slot] = py;
       out.s[slot] = s;
-      out.id[slot] = id;
-    }
-  }
-}
-
-// New particles of species A with ids id0 .. id0 + m - 1, uniform in the
-// rectangle [x0, x0 + wx) x [-1/2, ny - 1/2), those inside a fiber dropped,
-// appended to `out`.
-__global__ void __launch_bounds__(kThreads)
-    rwpt_spawn_kernel(const Args a, Buf out, unsigned long long *cnt, int kout,
-                      long long cap, long long t, unsigned long long id0,
-                      long long m, double x0, double wx) {
-  const long long stride = static_cast<long long>(gridDim.x) * blockDim.x;
-  for (long long base = static_cast<long long>(blockIdx.x) * blockDim.x; base < m;
-       base += stride) {
-    const long long j = base + threadIdx.x;
-    bool keep = j < m;
-    double px = 0.0, py = 0.0;
-    const unsigned long long id = id0 + static_cast<unsigned long long>(j);
-    if (keep) {
-      const unsigned long long ps = particle_seed(a.seed, id);
-      px = dadd(x0, dmul(wx, draw(ps, t, kSpawnDraw)));
-      py = dadd(-0.5, dmul(static_cast<double>(a.ny), draw(ps, t, kSpawnDraw + 1)));
-      for (int k = 0; k < a.nfib && keep; ++k) {
-        const Fiber &f = a.fib[k];
-        const double dx = dsub(px, f.cx), dy = dsub(py, f.cy);
-        if (dadd(dmul(dx, dx), dmul(dy, dy)) < dmul(f.rp, f.rp)) keep = false;
-      }
-    }
-    const long long slot = warp_slot(keep, cnt + kout, cap, cnt + kOverflow);
-    if (slot >= 0) {
-      out.x[slot] = px;
-      out.y[slot] = py;
-      out.s[slot] = 0;
       out.id[slot] = id;
     }
   }
@@ -350,6 +497,7 @@ struct lbm_rwpt {
   Buf buf[2];
   unsigned long long *cnt = nullptr;
   int cur = 0;                 // buffer holding the current particles
+  int count = 0;               // which of the three counts is theirs
   long long steps = 0, window = 0;
   unsigned long long next_id = 0;
   long long seed_count = 0;    // entrance particles per step
@@ -360,7 +508,7 @@ struct lbm_rwpt {
 namespace {
 
 struct RwptLayout {
-  size_t xy, id, s, fib, cnt, total;
+  size_t xy, id, s, fib, near, cnt, total;
 };
 RwptLayout rwpt_layout(long long cap, int nfib) {
   RwptLayout l{};
@@ -368,8 +516,9 @@ RwptLayout rwpt_layout(long long cap, int nfib) {
   l.id = a256(8 * static_cast<size_t>(cap));
   l.s = a256(4 * static_cast<size_t>(cap));
   l.fib = a256(sizeof(Fiber) * static_cast<size_t>(nfib > 0 ? nfib : 1));
+  l.near = a256(sizeof(Near) * static_cast<size_t>(nfib > 0 ? nfib : 1));
   l.cnt = a256(8 * kCounters);
-  l.total = 2 * (2 * l.xy + l.id + l.s) + l.fib + l.cnt;
+  l.total = 2 * (2 * l.xy + l.id + l.s) + l.fib + l.near + l.cnt;
   return l;
 }
 
@@ -421,6 +570,7 @@ extern "C" lbm_status lbm_rwpt_create(int32_t nx, int32_t ny,
     return LBM_ENOMEM;
   }
   std::vector<Fiber> fib(static_cast<size_t>(nfibers));
+  std::vector<Near> near(static_cast<size_t>(nfibers));
   for (int f = 0; f < nfibers; ++f) {
     const double *r = fibers + 6 * static_cast<int64_t>(f);
     const int cat = static_cast<int>(r[3]);
@@ -448,6 +598,15 @@ extern "C" lbm_status lbm_rwpt_create(int32_t nx, int32_t ny,
       q.nx = std::cos(r[4]);
       q.ny = std::sin(r[4]);
     }
+    // A point held by the fiber has coordinates of at most |c| + reach, so
+    // rounding it and the centre to float and subtracting is off by less
+    // than 1.2e-7 (|c| + reach) in each coordinate; the slack is three times
+    // that.  (Infinities and NaN leave the fiber in the double test.)
+    const double reach = std::fabs(q.rp) + p->delta;
+    const double d = reach + 1e-3 +
+                     4e-7 * (std::fabs(q.cx) + std::fabs(q.cy) + 2.0 * reach);
+    near[f] = {static_cast<float>(q.cx), static_cast<float>(q.cy),
+               static_cast<float>(1.00001 * d * d), 0.0f};
   }
   lbm_rwpt *r = new (std::nothrow) lbm_rwpt;
   if (!r) {
@@ -463,7 +622,9 @@ extern "C" lbm_status lbm_rwpt_create(int32_t nx, int32_t ny,
     r->buf[k].s = reinterpret_cast<int *>(o + 2 * l.xy + l.id);
   }
   Fiber *d_fib = reinterpret_cast<Fiber *>(b + 2 * (2 * l.xy + l.id + l.s));
-  r->cnt = reinterpret_cast<unsigned long long *>(b + 2 * (2 * l.xy + l.id + l.s) + l.fib);
+  Near *d_near = reinterpret_cast<Near *>(b + 2 * (2 * l.xy + l.id + l.s) + l.fib);
+  r->cnt = reinterpret_cast<unsigned long long *>(
+      b + 2 * (2 * l.xy + l.id + l.s) + l.fib + l.near);
   r->p = *p;
   r->nx = nx;
   r->ny = ny;
@@ -484,6 +645,8 @@ extern "C" lbm_status lbm_rwpt_create(int32_t nx, int32_t ny,
   a.seed = p->seed;
   a.u = static_cast<const double *>(u);
   a.fib = d_fib;
+  a.near = d_near;
+  a.plain = a.len > 1e-100 && a.len < 1e100 ? 0 : 1;
   r->seed_count = periodic ? 0 : static_cast<long long>(std::llround(p->density * ny));
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
@@ -492,6 +655,8 @@ extern "C" lbm_status lbm_rwpt_create(int32_t nx, int32_t ny,
   cudaError_t e = cudaSuccess;
   if (nfibers > 0)
     e = cudaMemcpy(d_fib, fib.data(), sizeof(Fiber) * fib.size(), cudaMemcpyHostToDevice);
+  if (nfibers > 0 && e == cudaSuccess)
+    e = cudaMemcpy(d_near, near.data(), sizeof(Near) * near.size(), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     delete r;
     return rfail("lbm_rwpt_create", e);
@@ -511,6 +676,7 @@ extern "C" lbm_status lbm_rwpt_init(lbm_rwpt *r, void *stream) {
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaMemsetAsync(r->cnt, 0, 8 * kCounters, st);
   r->cur = 0;
+  r->count = 0;
   r->steps = 0;
   r->window = 0;
   r->next_id = 0;
@@ -518,7 +684,7 @@ extern "C" lbm_status lbm_rwpt_init(lbm_rwpt *r, void *stream) {
   const long long m = std::llround(r->p.density * static_cast<double>(r->nx) * r->ny);
   if (e == cudaSuccess && m > 0) {
     rwpt_spawn_kernel<<<r->grid, kThreads, 0, st>>>(
-        r->a, r->buf[0], r->cnt, kCount0, r->cap, -1, 0ull, m, -0.5,
+        r->a, r->buf[0], r->cnt, kCount, r->cap, -1, 0ull, m, -0.5,
         static_cast<double>(r->nx));
     e = cudaGetLastError();
   }
@@ -537,20 +703,18 @@ extern "C" lbm_status lbm_rwpt_run(lbm_rwpt *r, int64_t nsteps, void *stream,
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaSuccess;
+  const long long entering = (r->seed_count + kThreads - 1) / kThreads;
+  const int spawners = static_cast<int>(entering < r->grid ? entering : r->grid);
   for (int64_t k = 0; k < nsteps && e == cudaSuccess; ++k) {
-    const int kin = kCount0 + r->cur, kout = kCount0 + (r->cur ^ 1);
-    e = cudaMemsetAsync(r->cnt + kout, 0, 8, st);
-    if (e != cudaSuccess) break;
-    rwpt_step_kernel<<<r->grid, kThreads, 0, st>>>(r->a, r->buf[r->cur],
-                                                   r->buf[r->cur ^ 1], r->cnt,
-                                                   kin, kout, r->cap, r->steps);
-    if (r->seed_count > 0)
-      rwpt_spawn_kernel<<<r->grid, kThreads, 0, st>>>(
-          r->a, r->buf[r->cur ^ 1], r->cnt, kout, r->cap, r->steps, r->next_id,
-          r->seed_count, -0.5, 1.0);
+    const int next = (r->count + 1) % 3;
+    rwpt_step_kernel<<<r->grid + spawners, kThreads, 0, st>>>(
+        r->a, r->buf[r->cur], r->buf[r->cur ^ 1], r->cnt, kCount + r->count,
+        kCount + next, kCount + (next + 1) % 3, r->cap, r->steps, r->next_id,
+        r->seed_count, r->grid);
     e = cudaGetLastError();
     r->next_id += static_cast<unsigned long long>(r->seed_count);
     r->cur ^= 1;
+    r->count = next;
     ++r->steps;
     ++r->window;
   }
@@ -563,8 +727,8 @@ extern "C" lbm_status lbm_rwpt_run(lbm_rwpt *r, int64_t nsteps, void *stream,
   std::memset(info, 0, sizeof(*info));
   info->steps = r->steps;
   info->window_steps = r->window;
-  info->alive = static_cast<int64_t>(h[kCount0 + r->cur]) < r->cap
-                    ? static_cast<int64_t>(h[kCount0 + r->cur])
+  info->alive = static_cast<int64_t>(h[kCount + r->count]) < r->cap
+                    ? static_cast<int64_t>(h[kCount + r->count])
                     : r->cap;
   for (int s = 0; s < 3; ++s) info->out[s] = static_cast<int64_t>(h[kOut + s]);
   info->overflow = h[kOverflow] ? 1 : 0;
@@ -603,7 +767,7 @@ extern "C" lbm_status lbm_rwpt_particles(lbm_rwpt *r, void *stream,
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   unsigned long long n = 0;
-  cudaError_t e = cudaMemcpyAsync(&n, r->cnt + kCount0 + r->cur, 8,
+  cudaError_t e = cudaMemcpyAsync(&n, r->cnt + kCount + r->count, 8,
                                   cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return rfail("lbm_rwpt_particles", e);
