@@ -65,7 +65,7 @@ void build_links(lbm_geometry *g) {
         word |= t << (4 * (j - 1));
       }
       g->links[n] = word;
-      if (word != 0u) g->bnodes.push_back(n);
+      if (word != 0u) g->bnodes.push_back({static_cast<uint32_t>(n), word});
     }
   }
   g->n_solid = nsol;

@@ -3,7 +3,7 @@
 
 namespace lbm {
 template cudaError_t launch_adr<PrecF32>(int, int, const AdrArgs &,
-                                            cudaStream_t, const AdrOverlap *);
+                                            cudaStream_t);
 template cudaError_t launch_adr_flux<PrecF32>(int, const void *, const RefT *,
                                                  const uint32_t *, long long,
                                                  int, int, int, double *,
@@ -13,6 +13,6 @@ template cudaError_t launch_flow<PrecF32>(int, const FlowArgs &, dim3,
 template cudaError_t launch_adjoint<PrecF32>(int, int, const AdjArgs &,
                                                 cudaStream_t);
 template cudaError_t launch_adjoint_grad<PrecF32>(
-    int, const AdjArgs &, const long long *, long long, const void *, double *,
+    int, const AdjArgs &, const BoundaryNode *, long long, const void *, double *,
     double *, const int32_t *, double *, double, double, cudaStream_t);
 }  // namespace lbm

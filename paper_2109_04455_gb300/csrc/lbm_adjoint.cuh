@@ -115,7 +115,7 @@ __device__ __forceinline__ void adj_eq(const AdjArgs &a, long long n, T (&E)[9])
     for (int i = 0; i < 9; ++i) E[i] = T(a.etab[(long long)i * a.plane + n]);
   } else {
     const T *U = static_cast<const T *>(a.u);
-    eq_factors<T>(U[n], U[a.plane + n], E);
+    eq_factors(U[n], U[a.plane + n], E);
   }
 }
 
@@ -194,13 +194,13 @@ __global__ void __launch_bounds__(kBlockX) adj_kernel(const AdjArgs a) {
 // and, when fiber ids are given, d eps/dw_f += k1 (first) - k2 (second).
 template <typename T, int NS>
 __global__ void __launch_bounds__(kBlockX)
-    adj_grad_kernel(const AdjArgs a, const long long *bnodes, long long nbnd,
+    adj_grad_kernel(const AdjArgs a, const BoundaryNode *bnodes, long long nbnd,
                     const T *conc, double *dkab, double *dkbc,
                     const int32_t *fiber, double *dw, double k1, double k2) {
   const long long t = (long long)blockIdx.x * kBlockX + threadIdx.x;
   if (t >= nbnd) return;
-  const long long n = bnodes[t];
-  const uint32_t lw = a.links[n];
+  const long long n = bnodes[t].n;
+  const uint32_t lw = bnodes[t].links;
   const int x = static_cast<int>(n % a.nx_pad);
   const int y = static_cast<int>(n / a.nx_pad);
   T mu[NS][9];

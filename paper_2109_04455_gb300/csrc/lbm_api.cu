@@ -131,7 +131,7 @@ extern "C" lbm_status lbm_geometry_upload(lbm_geometry *g, void *dev_ws,
     e = cudaMemcpyAsync(d_kab, g->kab.data(), 8 * p, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_kbc, g->kbc.data(), 8 * p, cudaMemcpyHostToDevice, st);
-  long long *d_bnodes = reinterpret_cast<long long *>(
+  BoundaryNode *d_bnodes = reinterpret_cast<BoundaryNode *>(
       b + align256(4 * p) + 2 * align256(8 * p));
   if (e == cudaSuccess && !g->bnodes.empty())
     e = cudaMemcpyAsync(d_bnodes, g->bnodes.data(), 8 * g->bnodes.size(),
@@ -310,7 +310,6 @@ struct lbm_adr_solver {
   int64_t steps = 0;
   bool has_check = false;
   long long nb = 0;
-  AdrOverlap ov;   // boundary kernel beside the bulk kernel
 };
 
 struct AdrLayout {
@@ -324,7 +323,7 @@ static AdrLayout adr_layout(const lbm_geometry *g, const lbm_adr_params *p) {
   l.buf = align256(ns * 9 * pl * store_bytes(p->precision));
   l.cprev = align256(ns * pl * compute_bytes(p->precision));
   l.partials = align256(static_cast<size_t>(adr_partial_rows(
-                            g->nx_pad, g->ny,
+                            p->precision, g->nx_pad, g->ny,
                             static_cast<long long>(g->bnodes.size()))) *
                         3 * ns * 8);
   l.scratch = align256(kReduceGrid * 3 * ns * 8);
@@ -354,11 +353,11 @@ extern "C" size_t lbm_adr_ws_bytes(const lbm_geometry *g,
 }
 
 static cudaError_t adr_launch(int prec, int ns, int mode, const AdrArgs &a,
-                              cudaStream_t st, const AdrOverlap *ov = nullptr) {
+                              cudaStream_t st) {
   switch (prec) {
-    case LBM_F64: return launch_adr<PrecF64>(ns, mode, a, st, ov);
-    case LBM_F32: return launch_adr<PrecF32>(ns, mode, a, st, ov);
-    default: return launch_adr<PrecF16Dev>(ns, mode, a, st, ov);
+    case LBM_F64: return launch_adr<PrecF64>(ns, mode, a, st);
+    case LBM_F32: return launch_adr<PrecF32>(ns, mode, a, st);
+    default: return launch_adr<PrecF16Dev>(ns, mode, a, st);
   }
 }
 
@@ -443,7 +442,7 @@ extern "C" lbm_status lbm_adr_create(const lbm_geometry *g,
     s->rbuf[0] = reinterpret_cast<RefT *>(rb);
     s->rbuf[1] = reinterpret_cast<RefT *>(rb + l.ref);
   }
-  s->nb = adr_partial_rows(g->nx_pad, g->ny,
+  s->nb = adr_partial_rows(p->precision, g->nx_pad, g->ny,
                            static_cast<long long>(g->bnodes.size()));
   AdrArgs &a = s->a;
   a.links = g->d_links;
@@ -455,7 +454,6 @@ extern "C" lbm_status lbm_adr_create(const lbm_geometry *g,
   a.partials = s->partials;
   a.bnodes = g->d_bnodes;
   a.nbnd = static_cast<long long>(g->bnodes.size());
-  a.part_off = 0;
   a.plane = plane_of(g);
   a.nx = g->nx;
   a.ny = g->ny;
@@ -469,29 +467,11 @@ extern "C" lbm_status lbm_adr_create(const lbm_geometry *g,
     a.fomega[k] = static_cast<float>(a.omega[k]);
     a.fcin[k] = static_cast<float>(a.cin[k]);
   }
-  // second stream for the boundary-node kernel (no device memory involved)
-  if (!g->bnodes.empty()) {
-    cudaError_t e = cudaStreamCreateWithFlags(&s->ov.aux, cudaStreamNonBlocking);
-    if (e == cudaSuccess)
-      e = cudaEventCreateWithFlags(&s->ov.fork, cudaEventDisableTiming);
-    if (e == cudaSuccess)
-      e = cudaEventCreateWithFlags(&s->ov.join, cudaEventDisableTiming);
-    if (e != cudaSuccess) {
-      lbm_adr_destroy(s);
-      return cuda_fail("lbm_adr_create", e);
-    }
-  }
   *out = s;
   return LBM_OK;
 }
 
-extern "C" void lbm_adr_destroy(lbm_adr_solver *s) {
-  if (!s) return;
-  if (s->ov.fork) cudaEventDestroy(s->ov.fork);
-  if (s->ov.join) cudaEventDestroy(s->ov.join);
-  if (s->ov.aux) cudaStreamDestroy(s->ov.aux);
-  delete s;
-}
+extern "C" void lbm_adr_destroy(lbm_adr_solver *s) { delete s; }
 
 extern "C" lbm_status lbm_adr_init(lbm_adr_solver *s, void *stream) {
   NvtxRange nvtx_range("lbm_adr_init");
@@ -531,7 +511,7 @@ static cudaError_t adr_step(lbm_adr_solver *s, int mode, cudaStream_t st) {
   a.step = static_cast<unsigned>(s->steps);
   s->cur ^= 1;
   ++s->steps;
-  return adr_launch(s->p.precision, s->p.nspecies, mode, a, st, &s->ov);
+  return adr_launch(s->p.precision, s->p.nspecies, mode, a, st);
 }
 
 extern "C" lbm_status lbm_adr_run(lbm_adr_solver *s, int64_t nsteps,

@@ -9,7 +9,7 @@
 // instance's check-step partial sums occupy a contiguous row range.  A
 // persistent grid of blocks walks the list; per item the instance's
 // arguments are staged in shared memory and the same per-node updates as the
-// single-lattice kernels run (adr_interior_node / adr_general_node), so a
+// single-lattice kernels run (adr_interior_node / adr_boundary_node), so a
 // batched solve gives the same populations as lbm_adr_solve on each lattice.
 #include <cuda_runtime.h>
 
@@ -90,9 +90,8 @@ __global__ void __launch_bounds__(BX)
       const long long t =
           static_cast<long long>(item & ((1ull << 48) - 1)) + threadIdx.x;
       if (t < sa.nbnd) {
-        const long long n = sa.bnodes[t];
-        adr_general_node<P, NS, MODE>(sa, n, static_cast<int>(n % sa.nx_pad),
-                                      sa.links[n], acc[0]);
+        const BoundaryNode b = sa.bnodes[t];
+        adr_boundary_node<P, NS, MODE>(sa, b.n, b.links, acc[0]);
       }
     }
     if constexpr (MODE == kAdrCheck)
@@ -528,7 +527,6 @@ extern "C" lbm_status lbm_batch_create(int32_t count,
     a.partials = nullptr;
     a.bnodes = g->d_bnodes;
     a.nbnd = static_cast<long long>(g->bnodes.size());
-    a.part_off = 0;
     a.plane = static_cast<long long>(g->nx_pad) * g->ny;
     a.nx = g->nx;
     a.ny = g->ny;

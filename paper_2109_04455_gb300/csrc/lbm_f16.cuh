@@ -128,15 +128,6 @@ __device__ __forceinline__ float2 push2(int i, float2 g, float2 e, const PushK2 
 #ifndef LBM_F16_SR
 #define LBM_F16_SR 1
 #endif
-// LBM_PAIR_PER_SPECIES = 1 (default): the bulk pair kernel loads each
-// species' 24 pairs just before that species' arithmetic, which needs 80
-// registers (6 blocks per SM) instead of 122 (4 blocks) for all 72 pairs
-// up front; with the L2 prefetch ahead the loads mostly hit L2, so the
-// shorter load phases and 50% more resident warps win (1.634 ms per step
-// of the 16384 x 4096 lattice against 1.692 ms).
-#ifndef LBM_PAIR_PER_SPECIES
-#define LBM_PAIR_PER_SPECIES 1
-#endif
 // Hash of (node pair, step) for the random bits.  Its constants are
 // published integer-hash multipliers: 0x9E3779B1 (2^32 divided by the golden
 // ratio, Knuth's multiplicative hashing), 0x85EBCA77 (the second 32-bit
@@ -252,8 +243,7 @@ __device__ __forceinline__ void adr_interior_node_f16(const AdrArgs &a, long lon
 // y +- 1 exist whenever either node is interior.  The reference
 // concentrations of the source nodes come the same way (three rows of three
 // pairs per species).  The arithmetic is that of adr_interior_node_f16.
-// Launched with kBlockX / 2 threads on the grid of adr_bulk_kernel, so a
-// block covers the same kBlockX nodes and writes the same partial-sum row.
+// A block has kBlockX / 2 threads and covers a segment of kBlockX nodes.
 //
 // Each thread reads 24 pairs per species: slot 0..8 its own pair of plane
 // i, 9..14 the side pair of the six planes with c_ix != 0 (directions 1, 3,
@@ -378,15 +368,12 @@ __device__ __forceinline__ void pair_update(const AdrArgs &a, int y, int x0,
   }
 }
 
-// The bulk kernel.  A block first sends the L2 prefetches for the block
-// LBM_PREFETCH_ROWS_F16 rows below it, then each thread loads its pairs
-// (per species by default, or all 24 x NS before any arithmetic with
-// LBM_PAIR_PER_SPECIES = 0) and updates its two nodes.  The check-step form
-// keeps its partial sums as well and is bounded at 5 blocks per SM (96
-// registers) so that it does not spill.
+// The two nodes per thread of one row segment, loaded species by species:
+// the block first sends the L2 prefetches for the segment
+// LBM_PREFETCH_ROWS_F16 rows below it.
 template <int NS, int MODE>
-__global__ void __launch_bounds__(kPairThreads, MODE == kAdrCheck ? 5 : LBM_PAIR_MIN_BLOCKS)
-    adr_bulk_pair_kernel(const AdrArgs a) {
+__device__ __forceinline__ void pair_segment(const AdrArgs &a,
+                                             float (&acc)[2][3 * NS]) {
   const int y = blockIdx.y;
   if (LBM_PREFETCH_ROWS_F16 > 0)
     bulk_prefetch_rows<__half, float, NS, true>(a, y + LBM_PREFETCH_ROWS_F16);
@@ -395,40 +382,37 @@ __global__ void __launch_bounds__(kPairThreads, MODE == kAdrCheck ? 5 : LBM_PAIR
   uint2 lw = make_uint2(kSolidNode, kSolidNode);
   if (x0 < a.nx_pad) lw = *reinterpret_cast<const uint2 *>(a.links + n0);
   const bool in0 = lw.x == 0u, in1 = lw.y == 0u;
+  if (!in0 && !in1) return;
+  const __half2 z2 = __float2half2_rn(0.0f);
+  const float *__restrict__ U = static_cast<const float *>(a.u);
+  const float2 ux = *reinterpret_cast<const float2 *>(U + n0);
+  const float2 uy = *reinterpret_cast<const float2 *>(U + a.plane + n0);
+  // each species' pairs are loaded as its arithmetic needs them (the stores
+  // of one species keep the next one's loads behind them)
+  pair_update<NS, MODE>(a, y, x0, in0, in1, ux, uy, [&](int s, int k) {
+    const PairSrc q = pair_src(a, s, k, y, x0, in0, in1);
+    return q.need ? *reinterpret_cast<const __half2 *>(q.p) : z2;
+  }, acc);
+}
+
+// The check step of the FP16 storage: the row segments two nodes per thread,
+// and the boundary chunks.  Bounded at 5 blocks per SM (96 registers), so
+// that it does not spill with its partial sums.
+template <int NS>
+__global__ void __launch_bounds__(kPairThreads, 5)
+    adr_check_pair_kernel(const AdrArgs a) {
   float acc[2][3 * NS];   // check-step values of node x0 and of node x0 + 1
 #pragma unroll
   for (int k = 0; k < 3 * NS; ++k) acc[0][k] = acc[1][k] = 0.0f;
-  if (in0 || in1) {
-    const __half2 z2 = __float2half2_rn(0.0f);
-    const float *__restrict__ U = static_cast<const float *>(a.u);
-    const float2 ux = *reinterpret_cast<const float2 *>(U + n0);
-    const float2 uy = *reinterpret_cast<const float2 *>(U + a.plane + n0);
-#if LBM_PAIR_PER_SPECIES
-    // each species' pairs are loaded as its arithmetic needs them (the
-    // stores of one species keep the next one's loads behind them)
-    pair_update<NS, MODE>(a, y, x0, in0, in1, ux, uy, [&](int s, int k) {
-      const PairSrc q = pair_src(a, s, k, y, x0, in0, in1);
-      return q.need ? *reinterpret_cast<const __half2 *>(q.p) : z2;
-    }, acc);
-#else
-    __half2 v[NS][kPairSlots];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) {
-#pragma unroll
-      for (int k = 0; k < kPairSlots; ++k) {
-        const PairSrc q = pair_src(a, s, k, y, x0, in0, in1);
-        v[s][k] = q.need ? *reinterpret_cast<const __half2 *>(q.p) : z2;
-      }
-    }
-    pair_update<NS, MODE>(a, y, x0, in0, in1, ux, uy,
-                          [&](int s, int k) { return v[s][k]; }, acc);
-#endif
-  }
-  if constexpr (MODE == kAdrCheck) {
-    const long long b = (long long)blockIdx.y * gridDim.x + blockIdx.x;
+  const long long chunk = boundary_chunk(a);
+  if (chunk >= 0)
+    boundary_nodes<PrecF16Dev, NS, kAdrCheck, kPairThreads>(a, chunk, acc[0]);
+  else
+    pair_segment<NS, kAdrCheck>(a, acc);
+  const long long row = partial_row<kPairThreads>(a, chunk);
+  if (row >= 0)
     block_partials_store<2 * NS, NS, 2, kPairThreads, float>(
-        acc, a.partials + b * (3 * NS));
-  }
+        acc, a.partials + row * (3 * NS));
 }
 
 // FP16 plain step, four nodes per thread: nodes x0 .. x0 + 3 (x0 a multiple
@@ -446,8 +430,7 @@ __global__ void __launch_bounds__(kPairThreads, MODE == kAdrCheck ? 5 : LBM_PAIR
 // (x0, x0 + 1) and (x0 + 2, x0 + 3), operation for operation (the same
 // packed roundings, the same random bits per pair), so every stored half is
 // the two-node kernel's.  Plain steps only: check steps keep the two-node
-// kernel, which also writes the partial sums.  Launched with kBlockX / 4
-// threads on the grid of adr_bulk_kernel.
+// kernel, which also writes the partial sums.
 #ifndef LBM_QUAD_MIN_BLOCKS
 #define LBM_QUAD_MIN_BLOCKS 8
 #endif
@@ -455,9 +438,15 @@ constexpr int kQuadThreads = kBlockX / 4;
 
 template <int NS>
 __global__ void __launch_bounds__(kQuadThreads, LBM_QUAD_MIN_BLOCKS)
-    adr_bulk_quad_kernel(const AdrArgs a) {
+    adr_step_quad_kernel(const AdrArgs a) {
   static_assert(kQuadThreads >= 9 * NS + NS + 3, "one prefetch per thread");
   static_assert(kQuadThreads % 32 == 0, "whole warps");
+  const long long chunk = boundary_chunk(a);
+  if (chunk >= 0) {
+    float acc[3 * NS];
+    boundary_nodes<PrecF16Dev, NS, kAdrStep, kQuadThreads>(a, chunk, acc);
+    return;
+  }
   const int y = blockIdx.y;
   if (LBM_PREFETCH_ROWS_F16 > 0)
     bulk_prefetch_rows<__half, float, NS, true>(a, y + LBM_PREFETCH_ROWS_F16);

@@ -32,6 +32,12 @@ constexpr uint32_t kSolidNode = 0xFFFFFFFFu;
 constexpr int kCx[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
 constexpr int kCy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
 
+// Entry of the boundary-node list: a fluid node with a non-zero link word
+// (node numbers fit 32 bits: 2^32 nodes would not fit the device).
+struct BoundaryNode {
+  uint32_t n, links;
+};
+
 inline int64_t pad32(int64_t n) { return (n + 31) / 32 * 32; }
 inline size_t align256(size_t n) { return (n + 255) / 256 * 256; }
 
@@ -73,14 +79,14 @@ struct lbm_geometry {
   std::vector<uint8_t> solid;     // [ny][nx]
   std::vector<double> kab, kbc;   // [ny][nx_pad]
   std::vector<uint32_t> links;    // [ny][nx_pad]
-  std::vector<long long> bnodes;  // fluid nodes with a non-zero link word
+  std::vector<lbm::BoundaryNode> bnodes;  // fluid nodes with a non-zero link word
   std::vector<int32_t> fiber;     // [ny][nx_pad] owning fiber, -1 elsewhere
   int32_t nfibers = 0;
   int32_t periodic = 0;           // LBM_PERIODIC_X | LBM_PERIODIC_Y
   double k1 = 0.0, k2 = 0.0;
   // device copies (borrowed from the caller's workspace after upload)
   const uint32_t *d_links = nullptr;
-  const long long *d_bnodes = nullptr;
+  const lbm::BoundaryNode *d_bnodes = nullptr;
   const double *d_kab = nullptr;
   const double *d_kbc = nullptr;
   bool uploaded = false;

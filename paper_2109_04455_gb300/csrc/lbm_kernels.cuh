@@ -25,31 +25,13 @@
 
 namespace lbm {
 
-// Launch shape of the lattice kernels (compile-time tuning knobs):
-//   LBM_BLOCK_X        threads per block = nodes of one row segment
-//   LBM_ADR_MIN_BLOCKS if defined, resident blocks per SM asked of the
-//                      register allocator for every precision (otherwise
-//                      each precision's kMinBlocks below)
+// Launch shape of the lattice kernels:
+//   LBM_BLOCK_X        threads per block = nodes of one row segment of the
+//                      flow, initial-state and adjoint kernels
 #ifndef LBM_BLOCK_X
 #define LBM_BLOCK_X 256
 #endif
-//   LBM_ADR_PAIR_F16   1: the FP16 bulk step updates two nodes per thread
-//                      (adr_bulk_pair_kernel); 0: one node per thread
-#ifndef LBM_ADR_PAIR_F16
-#define LBM_ADR_PAIR_F16 1
-#endif
-//   LBM_PAIR_MIN_BLOCKS resident blocks per SM asked of the register
-//                      allocator for adr_bulk_pair_kernel (6: 80 registers
-//                      with per-species loads)
-#ifndef LBM_PAIR_MIN_BLOCKS
-#define LBM_PAIR_MIN_BLOCKS 6
-#endif
 constexpr int kBlockX = LBM_BLOCK_X;
-#ifdef LBM_ADR_MIN_BLOCKS
-#define LBM_MIN_BLOCKS(P) LBM_ADR_MIN_BLOCKS
-#else
-#define LBM_MIN_BLOCKS(P) P::kMinBlocks
-#endif
 constexpr int kReduceThreads = 256;
 
 // ---------------------------------------------------------------------------
@@ -59,7 +41,7 @@ struct PrecF64 {
   using S = double;
   using T = double;
   static constexpr bool kDev = false;
-  static constexpr int kMinBlocks = 1;
+  static constexpr int kMinBlocks = 2;   // <= 128 registers
   static __device__ __forceinline__ T load(S v) { return v; }
   static __device__ __forceinline__ S store(T v) { return v; }
 };
@@ -67,7 +49,7 @@ struct PrecF32 {
   using S = float;
   using T = float;
   static constexpr bool kDev = false;
-  static constexpr int kMinBlocks = 1;
+  static constexpr int kMinBlocks = 4;   // <= 64 registers
   static __device__ __forceinline__ T load(S v) { return v; }
   static __device__ __forceinline__ S store(T v) { return v; }
 };
@@ -82,7 +64,6 @@ struct PrecF16Dev {
   using S = __half;
   using T = float;
   static constexpr bool kDev = true;
-  static constexpr int kMinBlocks = 5;   // <= 51 registers, 40 warps per SM
   static __device__ __forceinline__ T load(S v) {
     return __half2float(v) * (1.0f / 16384.0f);
   }
@@ -243,6 +224,31 @@ template <>
 __device__ __forceinline__ float pick<float>(double, float f) { return f; }
 
 
+// Every operation of the update is written with an explicit rounding (no
+// contraction is left to the compiler): the two-step kernel, the one-step
+// kernel, the boundary nodes, the batch kernel and the FP64 table must get
+// the same bits for the same node, so that a run's result depends neither on
+// how its steps are grouped into launches nor on the batch it is part of.
+__device__ __forceinline__ float fma_rn(float x, float y, float z) { return __fmaf_rn(x, y, z); }
+__device__ __forceinline__ double fma_rn(double x, double y, double z) { return __fma_rn(x, y, z); }
+__device__ __forceinline__ float mul_rn(float x, float y) { return __fmul_rn(x, y); }
+__device__ __forceinline__ double mul_rn(double x, double y) { return __dmul_rn(x, y); }
+__device__ __forceinline__ float add_rn(float x, float y) { return __fadd_rn(x, y); }
+__device__ __forceinline__ double add_rn(double x, double y) { return __dadd_rn(x, y); }
+// sum of a node's nine populations
+template <typename T>
+__device__ __forceinline__ T sum_rn(const T (&g)[9]) {
+  T c = g[0];
+#pragma unroll
+  for (int i = 1; i < 9; ++i) c = add_rn(c, g[i]);
+  return c;
+}
+// BGK relaxation of a population g towards c E
+template <typename T>
+__device__ __forceinline__ T relax(T om, T c, T E, T g) {
+  return fma_rn(om, fma_rn(c, E, -g), g);
+}
+
 // ---------------------------------------------------------------------------
 // ADR
 // ---------------------------------------------------------------------------
@@ -254,11 +260,12 @@ struct AdrArgs {
   const void *u;            // T [2][plane]
   void *cprev;              // T [ns][plane]     (check steps)
   double *partials;         // [rows][3*ns]      (check steps)
-  const long long *bnodes;  // boundary fluid nodes (link word != 0)
+  const BoundaryNode *bnodes;  // boundary fluid nodes (link word != 0)
   long long nbnd;           // number of boundary nodes
-  long long part_off;       // first partial row of the boundary kernel
   long long plane;          // ny * nx_pad
   int nx, ny, nx_pad;
+  int nxb;                  // row segments of a step's grid; blockIdx.x
+                            // beyond them takes boundary-node chunks
   int abb_all;              // anti-bounce-back inlet for every species
   int nodewise;             // every population of a reactive node reacts
   unsigned step;            // steps done before this one (rounding seed)
@@ -280,58 +287,24 @@ struct AdrArgs {
 enum AdrMode { kAdrStep = 0, kAdrCheck = 1, kAdrInit = 2 };
 
 
-// value added back to the stored population (s, i) of node m (half storage
-// only: w_i times the node's reference concentration)
-template <class P>
-__device__ __forceinline__ typename P::T adr_ref(const AdrArgs &a, int s, int i,
-                                                 long long m) {
-  using T = typename P::T;
-  if constexpr (P::kDev)
-    return Lattice<T>::w(i) * T(ref_get(a.rsrc, s * a.plane + m));
-  else
-    return T(0);
-}
-// value removed before storing population i of a node whose reference is c
-template <class P>
-__device__ __forceinline__ typename P::T adr_unref(int i, typename P::T c) {
-  using T = typename P::T;
-  if constexpr (P::kDev)
-    return Lattice<T>::w(i) * c;
-  else
-    return T(0);
-}
-
-template <class P>
-__device__ __forceinline__ typename P::T adr_ld(const AdrArgs &a, int s, int i,
-                                                long long m) {
-  const typename P::S *src = static_cast<const typename P::S *>(a.src);
-  return P::load(src[(long long)(s * 9 + i) * a.plane + m]) + adr_ref<P>(a, s, i, m);
-}
-
 // equilibrium factors E_i(u), shared by every species:
 // g_i^eq = C * E_i, E_i = w_i (1 + 3 c.u + 4.5 (c.u)^2 - 1.5 u.u)
-template <typename T>
-__device__ __forceinline__ void eq_factors(T ux, T uy, T (&E)[9]) {
-  const T uu = ux * ux + uy * uy;
+__device__ __forceinline__ void eq_factors(float ux, float uy, float (&E)[9]) {
+  const float uu = fma_rn(ux, ux, mul_rn(uy, uy));
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
-    const T cu = T(cx(i)) * ux + T(cy(i)) * uy;
-    E[i] = Lattice<T>::w(i) * (T(1) + T(3) * cu + T(4.5) * cu * cu - T(1.5) * uu);
+    const float cu = add_rn(float(cx(i)) * ux, float(cy(i)) * uy);
+    E[i] = mul_rn(Lattice<float>::w(i),
+                  fma_rn(-1.5f, uu, fma_rn(mul_rn(4.5f, cu), cu, fma_rn(3.0f, cu, 1.0f))));
   }
 }
-// The double version is written with explicit roundings: the FP64 step reads
-// E from a table that eq_table_kernel fills once per solver, while boundary
-// nodes and the batch kernel compute it in place, and all of them must get
-// the same bits.
-template <>
-__device__ __forceinline__ void eq_factors<double>(double ux, double uy,
-                                                   double (&E)[9]) {
-  const double base = __fma_rn(-1.5, __fma_rn(ux, ux, __dmul_rn(uy, uy)), 1.0);
+__device__ __forceinline__ void eq_factors(double ux, double uy, double (&E)[9]) {
+  const double base = fma_rn(-1.5, fma_rn(ux, ux, mul_rn(uy, uy)), 1.0);
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
-    const double cu = __dadd_rn(double(cx(i)) * ux, double(cy(i)) * uy);
-    E[i] = __dmul_rn(Lattice<double>::w(i),
-                     __fma_rn(__dmul_rn(4.5, cu), cu, __fma_rn(3.0, cu, base)));
+    const double cu = add_rn(double(cx(i)) * ux, double(cy(i)) * uy);
+    E[i] = mul_rn(Lattice<double>::w(i),
+                  fma_rn(mul_rn(4.5, cu), cu, fma_rn(3.0, cu, base)));
   }
 }
 
@@ -348,7 +321,7 @@ __device__ __forceinline__ void adr_eq(const AdrArgs &a, long long n,
     }
   }
   const T *__restrict__ U = static_cast<const T *>(a.u);
-  eq_factors<T>(U[n], U[a.plane + n], E);
+  eq_factors(U[n], U[a.plane + n], E);
 }
 
 // E_i(u) of every node of the lattice into etab [9][plane] (FP64 only)
@@ -358,7 +331,7 @@ __global__ void __launch_bounds__(256)
   const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= plane) return;
   T E[9];
-  eq_factors<T>(u[n], u[plane + n], E);
+  eq_factors(u[n], u[plane + n], E);
 #pragma unroll
   for (int i = 0; i < 9; ++i) etab[(long long)i * plane + n] = E[i];
 }
@@ -368,156 +341,187 @@ __global__ void __launch_bounds__(256)
 // C_B), so every source term is known when its species is collided, and only
 // one species' nine populations need to be live at a time.
 
-// Boundary node x (link word lw != 0), species s: replace every population
-// whose pull source is not a fluid node by the rule of that source's link
-// type (Eq. BC and bounce-back), reading the node's own post-collision values.
+// Where the update of a boundary node reads the old populations: the global
+// planes.  at(i, j, t) is the place of population i of the neighbour x + c_j
+// (j = 0: the node itself) across a link of type t (kFluid or kPeriodic),
+// get(s, place) its value for species s.  (The two-step kernel has another.)
 template <class P>
-__device__ __forceinline__ void adr_boundary(const AdrArgs &a, int s,
-                                             uint32_t lw, long long n, int x,
-                                             typename P::T (&g)[9]) {
+struct GlobalSource {
   using T = typename P::T;
-  T cb = T(0);
-  if (x == a.nx - 1) {
-#pragma unroll
-    for (int j = 0; j < 9; ++j) cb += adr_ld<P>(a, s, j, n);
+  struct Place {
+    long long plane, node;   // i * plane, node index
+    int i;
+  };
+  const AdrArgs &a;
+  long long n;
+  int x, y;
+  __device__ __forceinline__ Place at(int i, int j, uint32_t t) const {
+    const long long np = a.nx_pad;
+    return {i * a.plane,
+            t == kPeriodic ? neighbour(x, y, j, a.nx, a.ny, np) : n + cy(j) * np + cx(j),
+            i};
   }
-#pragma unroll
-  for (int i = 1; i < 9; ++i) {
-    const uint32_t t = nib(lw, opp(i));
-    if (t == kFluid || t == kPeriodic) continue;   // pulled already
-    const T back = adr_ld<P>(a, s, opp(i), n);
-    if (t == kInlet) {
-      g[i] = (s == 0 || a.abb_all)
-                 ? -back + T(2) * Lattice<T>::w(i) * pick<T>(a.cin[s], a.fcin[s])
-                                   : back;
-    } else if (t == kOutlet) {
-      g[i] = -back + T(2) * Lattice<T>::w(i) * cb;
-    } else {  // wall, inert or catalytic fiber: bounce-back
-      g[i] = back;
+  __device__ __forceinline__ T get(int s, const Place &k) const {
+    const typename P::S *src = static_cast<const typename P::S *>(a.src);
+    const typename P::S v = src[s * 9 * a.plane + k.plane + k.node];
+    if constexpr (P::kDev) {   // plus w_i times the node's reference
+      const T w = k.i == 0 ? Lattice<T>::w(0) : k.i < 5 ? Lattice<T>::w(1) : Lattice<T>::w(5);
+      return fma_rn(__half2float(v), 1.0f / 16384.0f,
+                    mul_rn(w, ref_get(a.rsrc, s * a.plane + k.node)));
+    } else {
+      return P::load(v);
     }
   }
+};
+
+// Source of species s on a population of weight w at rates ka, kb:
+//   Q_A = -k_AB w C_A,  Q_B = +k_AB w C_A - k_BC w C_B,  Q_C = +k_BC w C_B.
+template <int NS, typename T>
+__device__ __forceinline__ T react(int s, T ka, T kb, T w, const T (&C)[NS], T g) {
+  if (s == 0) return fma_rn(-mul_rn(ka, w), C[0], g);
+  const T cb = C[NS >= 2 ? 1 : 0];
+  if (s == 2) return fma_rn(mul_rn(kb, w), cb, g);
+  if (NS == 2) return fma_rn(mul_rn(ka, w), C[0], g);
+  return add_rn(g, fma_rn(mul_rn(ka, w), C[0], -mul_rn(mul_rn(kb, w), cb)));
 }
 
-// BGK collision of species s towards C E_i, then its Dawson source on links
-// into catalytic fiber nodes (Eq. source_lbm):
-//   Q_A = -k_AB w C_A,  Q_B = +k_AB w C_A - k_BC w C_B,  Q_C = +k_BC w C_B.
-// With a.nodewise, a node with catalytic links reacts on all nine
-// populations instead, with the mean rates of those links.
-// C[] holds the pre-collision concentrations of species 0..s; returns C_s.
-template <class P, int NS>
-__device__ __forceinline__ typename P::T adr_collide(const AdrArgs &a, int s,
-                                                     uint32_t lw, long long n,
-                                                     int x, int y,
-                                                     const typename P::T (&E)[9],
-                                                     typename P::T (&g)[9],
-                                                     typename P::T (&C)[NS]) {
-  using T = typename P::T;
-  T c = T(0);
-#pragma unroll
-  for (int i = 0; i < 9; ++i) c += g[i];
-  C[s] = c;
-  const T om = pick<T>(a.omega[s], a.fomega[s]);
-#pragma unroll
-  for (int i = 0; i < 9; ++i) g[i] = g[i] + om * (c * E[i] - g[i]);
-  if (lw != 0u && a.nodewise) {
-    const long long np = a.nx_pad;
+// The source of species s of a node with catalytic links: rates ka, kb of
+// the links, concentrations C of species 0..s.
+template <int NS, typename T>
+__device__ __forceinline__ void add_source(const AdrArgs &a, int s, uint32_t lw,
+                                           const T (&ka)[9], const T (&kb)[9],
+                                           const T (&C)[NS], T (&g)[9]) {
+  if (a.nodewise) {
     T sa = T(0), sb = T(0);
     int ncat = 0;
 #pragma unroll
     for (int j = 1; j < 9; ++j) {
       if (nib(lw, j) != kCat) continue;
-      const long long m = neighbour(x, y, j, a.nx, a.ny, np);
-      sa += T(a.kab[m]);
-      sb += T(a.kbc[m]);
+      sa = add_rn(sa, ka[j]);
+      sb = add_rn(sb, kb[j]);
       ++ncat;
     }
-    if (ncat > 0) {
-      const T ka = sa / T(ncat), kb = sb / T(ncat);
+    const T ma = sa / T(ncat), mb = sb / T(ncat);
 #pragma unroll
-      for (int i = 0; i < 9; ++i) {
-        const T wi = Lattice<T>::w(i);
-        if (s == 0) {
-          g[i] -= ka * wi * C[0];
-        } else if (s == 1) {
-          const T ra = ka * wi * C[0];
-          const T rb = (NS >= 3) ? kb * wi * C[NS >= 2 ? 1 : 0] : T(0);
-          g[i] += ra - rb;
-        } else {
-          g[i] += kb * wi * C[NS >= 2 ? 1 : 0];
-        }
-      }
-    }
-  } else if (lw != 0u) {
+    for (int i = 0; i < 9; ++i) g[i] = react<NS>(s, ma, mb, Lattice<T>::w(i), C, g[i]);
+  } else {
+#pragma unroll
+    for (int j = 1; j < 9; ++j)
+      if (nib(lw, j) == kCat) g[j] = react<NS>(s, ka[j], kb[j], Lattice<T>::w(j), C, g[j]);
+  }
+}
+
+// Update of a boundary node (x, y) (a fluid node with link word lw != 0): the
+// pulls, with the rule of the link's type wherever the source x - c_i is not
+// a fluid node (Eq. BC and bounce-back: all of them read the node's own
+// opposite population), BGK towards C E_i, then the Dawson source on links
+// into catalytic fiber nodes (Eq. source_lbm), or, with a.nodewise, on all
+// nine populations with the mean rates of those links.  put(s, g, c) stores
+// the new populations of species s.
+//
+// The node's latency bounds the step of a small lattice (a 200 x 100 one took
+// 23 us per step with each load behind its link's branch, species after
+// species), so every load is issued before any arithmetic: there is exactly
+// one per population, whatever the link types, from a selected place.
+template <int NS, class Src, typename T, class Put>
+__device__ __forceinline__ void boundary_update(const AdrArgs &a, const Src &src,
+                                                uint32_t lw, int x, int y,
+                                                const T (&E)[9], Put &&put) {
+  T g[NS][9], cb[NS], ka[9], kb[9];
+  bool outlet = false, cat = false;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    const uint32_t t = i == 0 ? (uint32_t)kFluid : nib(lw, opp(i));
+    const bool pulled = t == kFluid || t == kPeriodic;
+    outlet = outlet || t == kOutlet;
+    cat = cat || t == kCat;
+    const auto from = pulled ? src.at(i, opp(i), t) : src.at(opp(i), 0, kFluid);
+#pragma unroll
+    for (int s = 0; s < NS; ++s) g[s][i] = src.get(s, from);
+  }
+  if (cat) {
     const long long np = a.nx_pad;
 #pragma unroll
     for (int j = 1; j < 9; ++j) {
-      if (nib(lw, j) != kCat) continue;
-      const long long m = neighbour(x, y, j, a.nx, a.ny, np);
-      const T wj = Lattice<T>::w(j);
-      if (s == 0) {
-        g[j] -= T(a.kab[m]) * wj * C[0];
-      } else if (s == 1) {
-        const T ra = T(a.kab[m]) * wj * C[0];
-        const T rb = (NS >= 3) ? T(a.kbc[m]) * wj * C[NS >= 2 ? 1 : 0] : T(0);
-        g[j] += ra - rb;
-      } else {
-        g[j] += T(a.kbc[m]) * wj * C[NS >= 2 ? 1 : 0];
-      }
+      const bool on = nib(lw, j) == kCat;
+      const long long m = on ? neighbour(x, y, j, a.nx, a.ny, np) : 0;
+      ka[j] = on ? T(a.kab[m]) : T(0);
+      kb[j] = on ? T(a.kbc[m]) : T(0);
     }
   }
-  return c;
-}
-
-// Update of one fluid node x = n % nx_pad with every link rule in place (or
-// its initial state): the species one after the other.
-template <class P, int NS, int MODE>
-__device__ __forceinline__ void adr_general_node(const AdrArgs &a, long long n,
-                                                 int x, uint32_t lw,
-                                                 typename P::T (&acc)[3 * NS]) {
-  using S = typename P::S;
-  using T = typename P::T;
-  const long long plane = a.plane;
-  S *__restrict__ dst = static_cast<S *>(a.dst);
-  const long long np = (long long)a.nx_pad;
-  const int y = lw != 0u ? static_cast<int>(n / np) : 0;
-  T E[9];
-  adr_eq<P>(a, n, E);
+  if (outlet) {   // C_w = the node's own concentration
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      T own[9];
+#pragma unroll
+      for (int j = 0; j < 9; ++j) own[j] = src.get(s, src.at(j, 0, kFluid));
+      cb[s] = sum_rn(own);
+    }
+  }
   T C[NS];
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
-    T g[9];
-    if (MODE == kAdrInit) {
-      const T c0 = (s == 0) ? T(1) : T(0);
 #pragma unroll
-      for (int i = 0; i < 9; ++i) g[i] = c0 * E[i];
-    } else {
+    for (int i = 1; i < 9; ++i) {
+      const uint32_t t = nib(lw, opp(i));
+      const T w2 = T(2) * Lattice<T>::w(i);
+      if (t == kInlet && (s == 0 || a.abb_all))
+        g[s][i] = fma_rn(w2, pick<T>(a.cin[s], a.fcin[s]), -g[s][i]);
+      else if (t == kOutlet)
+        g[s][i] = fma_rn(w2, cb[s], -g[s][i]);
+    }
+    const T c = sum_rn(g[s]);
+    C[s] = c;
+    const T om = pick<T>(a.omega[s], a.fomega[s]);
 #pragma unroll
-      for (int i = 0; i < 9; ++i) {
-        // pull from x - c_i when that node is fluid (always for lw == 0),
-        // from the wrapped node across a periodic edge
-        const uint32_t t = (i == 0 || lw == 0u) ? (uint32_t)kFluid : nib(lw, opp(i));
-        if (t == kFluid)
-          g[i] = adr_ld<P>(a, s, i, n - (cy(i) * np + cx(i)));
-        else if (t == kPeriodic)
-          g[i] = adr_ld<P>(a, s, i, neighbour(x, y, opp(i), a.nx, a.ny, np));
-      }
-      if (lw != 0u) adr_boundary<P>(a, s, lw, n, x, g);
-    }
-    const T c = adr_collide<P, NS>(a, s, lw, n, x, y, E, g, C);
-    T cq = c;   // the reference stored with the populations (half path)
-    if constexpr (P::kDev) {
-      cq = ref_round(c);
-      a.rdst[s * plane + n] = __float2half_rn(c);
-    }
-#pragma unroll
-    for (int i = 0; i < 9; ++i)
-      dst[(long long)(s * 9 + i) * plane + n] = P::store(g[i] - adr_unref<P>(i, cq));
-    if (MODE == kAdrCheck) {
-      T *cp = static_cast<T *>(a.cprev);
-      check_add<NS, T>(acc, s, c, cp[s * plane + n]);
-      cp[s * plane + n] = c;
-    }
+    for (int i = 0; i < 9; ++i) g[s][i] = relax(om, c, E[i], g[s][i]);
+    if (cat) add_source<NS>(a, s, lw, ka, kb, C, g[s]);
+    put(s, g[s], c);
   }
+}
+
+// Store of the new populations of species s of node n, whose concentration
+// is c, in the global planes (half storage: less w_i times the reference,
+// which is stored beside them).
+template <class P, typename T>
+__device__ __forceinline__ void put_node(const AdrArgs &a, int s, long long n,
+                                         const T (&g)[9], T c) {
+  typename P::S *__restrict__ dst = static_cast<typename P::S *>(a.dst);
+  T cq = c;
+  if constexpr (P::kDev) {
+    cq = ref_round(c);
+    a.rdst[s * a.plane + n] = __float2half_rn(c);
+  }
+#pragma unroll
+  for (int i = 0; i < 9; ++i)
+    dst[(long long)(s * 9 + i) * a.plane + n] =
+        P::store(P::kDev ? fma_rn(-Lattice<T>::w(i), cq, g[i]) : g[i]);
+}
+
+// A boundary node of the global planes, link word lw.
+template <class P, int NS, int MODE>
+__device__ __forceinline__ void adr_boundary_node(const AdrArgs &a, long long n,
+                                                  uint32_t lw,
+                                                  typename P::T (&acc)[3 * NS]) {
+  using T = typename P::T;
+  const int y = static_cast<int>(n / a.nx_pad);
+  const int x = static_cast<int>(n - (long long)y * a.nx_pad);
+  T prev[NS];
+  T *cp = static_cast<T *>(a.cprev);
+  if (MODE == kAdrCheck) {
+#pragma unroll
+    for (int s = 0; s < NS; ++s) prev[s] = cp[s * a.plane + n];
+  }
+  T E[9];
+  adr_eq<P>(a, n, E);
+  boundary_update<NS>(a, GlobalSource<P>{a, n, x, y}, lw, x, y, E,
+                      [&](int s, const T (&g)[9], T c) {
+    put_node<P>(a, s, n, g, c);
+    if (MODE == kAdrCheck) {
+      check_add<NS, T>(acc, s, c, prev[s]);
+      cp[s * a.plane + n] = c;
+    }
+  });
 }
 
 // L2 prefetch ahead of the bulk stencil.  With D = LBM_PREFETCH_ROWS_* > 0
@@ -570,6 +574,34 @@ __device__ __forceinline__ void bulk_prefetch_rows(const AdrArgs &a, int yp) {
   }
 }
 
+// Boundary-node chunk of a step's grid.  A step is one launch: the blocks of
+// blockIdx.x < a.nxb update the interior nodes (link word 0) of one row
+// segment each, and those beyond take chunks of BX entries of the
+// boundary-node list with every link rule in place (both read only the old
+// populations and write disjoint nodes).  The chunk is the block's number
+// among the latter, spread over the rows; -1 for an interior block.  Two
+// launches on two streams, forked and joined by events every step, cost a
+// 1000 x 300 lattice 34 us per step, almost all of it host time.
+__device__ __forceinline__ long long boundary_chunk(const AdrArgs &a) {
+  return static_cast<int>(blockIdx.x) < a.nxb
+             ? -1
+             : (long long)(blockIdx.x - a.nxb) * gridDim.y + blockIdx.y;
+}
+template <class P, int NS, int MODE, int BX>
+__device__ __forceinline__ void boundary_nodes(const AdrArgs &a, long long chunk,
+                                               typename P::T (&acc)[3 * NS]) {
+  const long long t = chunk * BX + threadIdx.x;
+  if (t >= a.nbnd) return;
+  const BoundaryNode b = a.bnodes[t];
+  adr_boundary_node<P, NS, MODE>(a, b.n, b.links, acc);
+}
+// check-step partial row of this block: interior blocks row by row, then the
+// boundary chunks that exist (-1 for a block with neither)
+template <int BX>
+__device__ __forceinline__ long long partial_row(const AdrArgs &a, long long chunk) {
+  if (chunk < 0) return (long long)blockIdx.y * a.nxb + blockIdx.x;
+  return chunk * BX < a.nbnd ? (long long)gridDim.y * a.nxb + chunk : -1;
+}
 
 }  // namespace lbm
 // FP16-deviation storage: interior update (one and two nodes per thread)
@@ -613,14 +645,11 @@ __device__ __forceinline__ void adr_interior_node(const AdrArgs &a, long long n,
   adr_eq<P>(a, n, E);
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
-    T c = T(0);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) c += g[s][i];
+    const T c = sum_rn(g[s]);
     const T om = pick<T>(a.omega[s], a.fomega[s]);
 #pragma unroll
     for (int i = 0; i < 9; ++i)
-      dst[(long long)(s * 9 + i) * plane + n] =
-          P::store(g[s][i] + om * (c * E[i] - g[s][i]));
+      dst[(long long)(s * 9 + i) * plane + n] = P::store(relax(om, c, E[i], g[s][i]));
     if (MODE == kAdrCheck) {
       check_add<NS, T>(acc, s, c, prev[s]);
       cp[s * plane + n] = c;
@@ -628,60 +657,65 @@ __device__ __forceinline__ void adr_interior_node(const AdrArgs &a, long long n,
   }
 }
 
-// One node per thread, every link rule handled in place.  LIST = false: the
-// whole lattice (initial state; also the plain one-kernel step).  LIST = true:
-// only the boundary nodes of a.bnodes, after the bulk kernel (below) has
-// updated the interior nodes; its partial sums go to rows a.part_off + block.
-template <class P, int NS, int MODE, bool LIST>
-__global__ void __launch_bounds__(kBlockX, LBM_MIN_BLOCKS(P))
-    adr_node_kernel(const AdrArgs a) {
+// Initial state g* of every node: C_A = 1, the others 0, at equilibrium, with
+// the source of step 0 on catalytic links.
+template <class P, int NS>
+__global__ void __launch_bounds__(kBlockX)
+    adr_init_kernel(const AdrArgs a) {
   using T = typename P::T;
-  long long n;
-  int x;
-  uint32_t lw;
-  if (LIST) {
-    const long long t = (long long)blockIdx.x * kBlockX + threadIdx.x;
-    n = t < a.nbnd ? a.bnodes[t] : 0;
-    x = static_cast<int>(n % a.nx_pad);
-    lw = t < a.nbnd ? a.links[n] : kSolidNode;
-  } else {
-    x = blockIdx.x * kBlockX + threadIdx.x;
-    n = (long long)blockIdx.y * a.nx_pad + x;
-    lw = (x < a.nx_pad) ? a.links[n] : kSolidNode;
-  }
-  T acc[1][3 * NS];
+  const int x = blockIdx.x * kBlockX + threadIdx.x, y = blockIdx.y;
+  const long long n = (long long)y * a.nx_pad + x;
+  const uint32_t lw = (x < a.nx_pad) ? a.links[n] : kSolidNode;
+  if (lw == kSolidNode) return;
+  T E[9], C[NS];
+  adr_eq<P>(a, n, E);
 #pragma unroll
-  for (int k = 0; k < 3 * NS; ++k) acc[0][k] = T(0);
-  if (lw != kSolidNode) adr_general_node<P, NS, MODE>(a, n, x, lw, acc[0]);
-  if constexpr (MODE == kAdrCheck) {
-    const long long b = LIST ? a.part_off + blockIdx.x
-                             : (long long)blockIdx.y * gridDim.x + blockIdx.x;
-    block_partials_store<2 * NS, NS, 1, kBlockX, T>(acc, a.partials + b * (3 * NS));
+  for (int s = 0; s < NS; ++s) {
+    T g[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) g[i] = mul_rn(s == 0 ? T(1) : T(0), E[i]);
+    const T c = sum_rn(g), om = pick<T>(a.omega[s], a.fomega[s]);
+    C[s] = c;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) g[i] = relax(om, c, E[i], g[i]);
+    T ka[9], kb[9];
+    bool cat = false;
+#pragma unroll
+    for (int j = 1; j < 9; ++j) {
+      if (nib(lw, j) != kCat) continue;
+      const long long m = neighbour(x, y, j, a.nx, a.ny, a.nx_pad);
+      ka[j] = T(a.kab[m]);
+      kb[j] = T(a.kbc[m]);
+      cat = true;
+    }
+    if (cat) add_source<NS>(a, s, lw, ka, kb, C, g);
+    put_node<P>(a, s, n, g, c);
   }
 }
 
-// Bulk step, one node per thread: the interior formula for the nodes whose
-// eight neighbours are all fluid (link word 0); every other node is left to
-// adr_node_kernel<..., LIST = true>, which runs beside it.
-template <class P, int NS, int MODE>
-__global__ void __launch_bounds__(kBlockX, LBM_MIN_BLOCKS(P))
-    adr_bulk_kernel(const AdrArgs a) {
+// One step (or check step), one node per thread.  On large lattices (BX =
+// 256) the interior update needs its warps in flight, so the registers that
+// the boundary update would like are bounded (P::kMinBlocks blocks per SM).
+template <class P, int NS, int MODE, int BX>
+__global__ void __launch_bounds__(BX, BX == 256 ? P::kMinBlocks : 1)
+    adr_step_kernel(const AdrArgs a) {
   using T = typename P::T;
-  if constexpr (std::is_same<typename P::S, float>::value && LBM_PREFETCH_ROWS_F32 > 0)
-    bulk_prefetch_rows<float, float, NS, false>(a, blockIdx.y + LBM_PREFETCH_ROWS_F32);
-  const int x = blockIdx.x * kBlockX + threadIdx.x;
-  const long long n = (long long)blockIdx.y * a.nx_pad + x;
-  const uint32_t lw = (x < a.nx_pad) ? a.links[n] : kSolidNode;
   T acc[1][3 * NS];
 #pragma unroll
   for (int k = 0; k < 3 * NS; ++k) acc[0][k] = T(0);
-  // (half storage: the references of the nine source nodes are read next
-  // to the populations; gathering them with warp shuffles instead measured
-  // slower, the shuffles keep the population loads from being issued early)
-  if (lw == 0u) adr_interior_node<P, NS, MODE>(a, n, acc[0]);
+  const long long chunk = boundary_chunk(a);
+  if (chunk >= 0) {
+    boundary_nodes<P, NS, MODE, BX>(a, chunk, acc[0]);
+  } else {
+    const int x = blockIdx.x * BX + threadIdx.x;
+    const long long n = (long long)blockIdx.y * a.nx_pad + x;
+    const uint32_t lw = (x < a.nx_pad) ? a.links[n] : kSolidNode;
+    if (lw == 0u) adr_interior_node<P, NS, MODE>(a, n, acc[0]);
+  }
   if constexpr (MODE == kAdrCheck) {
-    const long long b = (long long)blockIdx.y * gridDim.x + blockIdx.x;
-    block_partials_store<2 * NS, NS, 1, kBlockX, T>(acc, a.partials + b * (3 * NS));
+    const long long row = partial_row<BX>(a, chunk);
+    if (row >= 0)
+      block_partials_store<2 * NS, NS, 1, BX, T>(acc, a.partials + row * (3 * NS));
   }
 }
 
@@ -883,43 +917,49 @@ __global__ void __launch_bounds__(kBlockX) flow_kernel(const FlowArgs a) {
 // ---------------------------------------------------------------------------
 // launchers (one translation unit per precision instantiates them)
 // ---------------------------------------------------------------------------
-// A time step is the bulk kernel (two nodes per thread, interior formula)
-// followed by the boundary kernel over the boundary-node list; with
-// LBM_ADR_SPLIT=0 it is the one-node kernel over the whole lattice instead.
-#ifndef LBM_ADR_SPLIT
-#define LBM_ADR_SPLIT 1
-#endif
-inline dim3 adr_bulk_grid(int nx_pad, int ny) {
-  const int per = kBlockX;
-  return dim3(static_cast<unsigned>((nx_pad + per - 1) / per),
-              static_cast<unsigned>(ny));
+// Threads per block of a step (= nodes of a row segment, and entries of a
+// boundary chunk).  FP32 and FP64: 256, or 64 where 256 would leave SMs
+// without a block or cover a quarter more than the row (152 SMs with at
+// least four blocks of 256 each; a 200 x 100 lattice has 100 such blocks).
+// FP16 storage: 256-node segments throughout, which its kernels cover with
+// 64 (plain) and 128 (check) threads.
+inline int adr_block_x(int prec, int nx_pad, int ny) {
+  if (prec == LBM_F16DEV) return kBlockX;
+  const long long seg = (nx_pad + 255) / 256;
+  return seg * ny < 4 * 152 || seg * 256 * 4 > 5LL * nx_pad ? 64 : 256;
+}
+// Grid of a step: nxb row segments per row, plus the columns of blocks that
+// take the boundary chunks of bthreads nodes.
+struct AdrGrid {
+  int nxb;            // row segments per row
+  long long chunks;   // boundary chunks
+  dim3 grid;
+};
+inline AdrGrid adr_grid(int nx_pad, int ny, long long nbnd, int bx, int bthreads) {
+  AdrGrid g;
+  g.nxb = (nx_pad + bx - 1) / bx;
+  g.chunks = (nbnd + bthreads - 1) / bthreads;
+  g.grid = dim3(static_cast<unsigned>(g.nxb + (g.chunks + ny - 1) / ny),
+                static_cast<unsigned>(ny));
+  return g;
 }
 inline dim3 adr_node_grid(int nx_pad, int ny) {
   return dim3(static_cast<unsigned>((nx_pad + kBlockX - 1) / kBlockX),
               static_cast<unsigned>(ny));
 }
-inline long long adr_list_blocks(long long nbnd) {
-  return (nbnd + kBlockX - 1) / kBlockX;
+// boundary entries per chunk of a check step
+inline int adr_check_threads(int prec, int nx_pad, int ny) {
+  return prec == LBM_F16DEV ? kPairThreads : adr_block_x(prec, nx_pad, ny);
 }
 // partial-sum rows written by one check step
-inline long long adr_partial_rows(int nx_pad, int ny, long long nbnd) {
-  if (!LBM_ADR_SPLIT) {
-    const dim3 g = adr_node_grid(nx_pad, ny);
-    return static_cast<long long>(g.x) * g.y;
-  }
-  const dim3 g = adr_bulk_grid(nx_pad, ny);
-  return static_cast<long long>(g.x) * g.y + adr_list_blocks(nbnd);
+inline long long adr_partial_rows(int prec, int nx_pad, int ny, long long nbnd) {
+  const AdrGrid g = adr_grid(nx_pad, ny, nbnd, adr_block_x(prec, nx_pad, ny),
+                             adr_check_threads(prec, nx_pad, ny));
+  return static_cast<long long>(g.nxb) * ny + g.chunks;
 }
 
-// second stream and fork / join events for running the boundary-node kernel
-// beside the bulk kernel (aux == nullptr: one stream)
-struct AdrOverlap {
-  cudaStream_t aux = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr;
-};
 template <class P>
-cudaError_t launch_adr(int ns, int mode, const AdrArgs &a, cudaStream_t st,
-                       const AdrOverlap *ov = nullptr);
+cudaError_t launch_adr(int ns, int mode, const AdrArgs &a, cudaStream_t st);
 template <class P>
 cudaError_t launch_adr_flux(int ns, const void *g, const RefT *ref,
                             const uint32_t *links, long long plane, int nx_pad,
@@ -933,7 +973,7 @@ cudaError_t launch_adjoint(int ns, int mode, const AdjArgs &a, cudaStream_t st);
 cudaError_t launch_eq_table(const double *u, long long plane, double *etab,
                             cudaStream_t st);
 template <class P>
-cudaError_t launch_adjoint_grad(int ns, const AdjArgs &a, const long long *bnodes,
+cudaError_t launch_adjoint_grad(int ns, const AdjArgs &a, const BoundaryNode *bnodes,
                                 long long nbnd, const void *conc, double *dkab,
                                 double *dkbc, const int32_t *fiber, double *dw,
                                 double k1, double k2, cudaStream_t st);

@@ -8,68 +8,44 @@
 namespace lbm {
 
 template <class P, int NS, int MODE>
-static void launch_bulk(const AdrArgs &a, dim3 bg, cudaStream_t st) {
-  if constexpr (P::kDev && LBM_ADR_PAIR_F16)
-    adr_bulk_pair_kernel<NS, MODE><<<bg, dim3(kPairThreads), 0, st>>>(a);
-  else
-    adr_bulk_kernel<P, NS, MODE><<<bg, dim3(kBlockX), 0, st>>>(a);
+static void launch_step(AdrArgs a, cudaStream_t st) {
+  if constexpr (P::kDev) {
+    constexpr int kThreads = MODE == kAdrCheck ? kPairThreads : kQuadThreads;
+    const AdrGrid g = adr_grid(a.nx_pad, a.ny, a.nbnd, kBlockX, kThreads);
+    a.nxb = g.nxb;
+    if constexpr (MODE == kAdrCheck)
+      adr_check_pair_kernel<NS><<<g.grid, kThreads, 0, st>>>(a);
+    else
+      adr_step_quad_kernel<NS><<<g.grid, kThreads, 0, st>>>(a);
+  } else {
+    const int bx = adr_block_x(sizeof(typename P::S) == 8 ? LBM_F64 : LBM_F32,
+                               a.nx_pad, a.ny);
+    const AdrGrid g = adr_grid(a.nx_pad, a.ny, a.nbnd, bx, bx);
+    a.nxb = g.nxb;
+    if (bx == 64)
+      adr_step_kernel<P, NS, MODE, 64><<<g.grid, 64, 0, st>>>(a);
+    else
+      adr_step_kernel<P, NS, MODE, 256><<<g.grid, 256, 0, st>>>(a);
+  }
 }
 
 template <class P, int NS>
-static cudaError_t launch_adr_ns(int mode, const AdrArgs &a, cudaStream_t st,
-                                 const AdrOverlap *ov) {
-  const dim3 block(kBlockX);
-  if (mode == kAdrInit) {
-    adr_node_kernel<P, NS, kAdrInit, false>
-        <<<adr_node_grid(a.nx_pad, a.ny), block, 0, st>>>(a);
-    return cudaGetLastError();
-  }
-  if (!LBM_ADR_SPLIT) {
-    if (mode == kAdrStep)
-      adr_node_kernel<P, NS, kAdrStep, false>
-          <<<adr_node_grid(a.nx_pad, a.ny), block, 0, st>>>(a);
-    else
-      adr_node_kernel<P, NS, kAdrCheck, false>
-          <<<adr_node_grid(a.nx_pad, a.ny), block, 0, st>>>(a);
-    return cudaGetLastError();
-  }
-  const dim3 bg = adr_bulk_grid(a.nx_pad, a.ny);
-  AdrArgs b = a;
-  b.part_off = static_cast<long long>(bg.x) * bg.y;
-  const unsigned lb = static_cast<unsigned>(adr_list_blocks(a.nbnd));
-  // The boundary nodes run on a second stream next to the bulk kernel when
-  // one is given: both read only the old populations and write disjoint
-  // nodes, so the few boundary blocks hide in the bulk kernel's time.
-  cudaStream_t sb = st;
-  cudaError_t e = cudaSuccess;
-  if (lb && ov && ov->aux) {
-    e = cudaEventRecord(ov->fork, st);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(ov->aux, ov->fork, 0);
-    if (e != cudaSuccess) return e;
-    sb = ov->aux;
-  }
-  if (mode == kAdrStep) {
-    if (lb) adr_node_kernel<P, NS, kAdrStep, true><<<lb, block, 0, sb>>>(b);
-    launch_bulk<P, NS, kAdrStep>(a, bg, st);
-  } else {
-    if (lb) adr_node_kernel<P, NS, kAdrCheck, true><<<lb, block, 0, sb>>>(b);
-    launch_bulk<P, NS, kAdrCheck>(a, bg, st);
-  }
-  e = cudaGetLastError();
-  if (e == cudaSuccess && sb != st) {
-    e = cudaEventRecord(ov->join, sb);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ov->join, 0);
-  }
-  return e;
+static cudaError_t launch_adr_ns(int mode, const AdrArgs &a, cudaStream_t st) {
+  if (mode == kAdrInit)
+    adr_init_kernel<P, NS><<<adr_node_grid(a.nx_pad, a.ny), kBlockX, 0, st>>>(a);
+  else if (mode == kAdrStep)
+    launch_step<P, NS, kAdrStep>(a, st);
+  else
+    launch_step<P, NS, kAdrCheck>(a, st);
+  return cudaGetLastError();
 }
 
 template <class P>
-cudaError_t launch_adr(int ns, int mode, const AdrArgs &a, cudaStream_t st,
-                       const AdrOverlap *ov) {
+cudaError_t launch_adr(int ns, int mode, const AdrArgs &a, cudaStream_t st) {
   switch (ns) {
-    case 1: return launch_adr_ns<P, 1>(mode, a, st, ov);
-    case 2: return launch_adr_ns<P, 2>(mode, a, st, ov);
-    case 3: return launch_adr_ns<P, 3>(mode, a, st, ov);
+    case 1: return launch_adr_ns<P, 1>(mode, a, st);
+    case 2: return launch_adr_ns<P, 2>(mode, a, st);
+    case 3: return launch_adr_ns<P, 3>(mode, a, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -132,14 +108,14 @@ cudaError_t launch_adjoint(int ns, int mode, const AdjArgs &a, cudaStream_t st) 
 }
 
 template <class P>
-cudaError_t launch_adjoint_grad(int ns, const AdjArgs &a, const long long *bnodes,
+cudaError_t launch_adjoint_grad(int ns, const AdjArgs &a, const BoundaryNode *bnodes,
                                 long long nbnd, const void *conc, double *dkab,
                                 double *dkbc, const int32_t *fiber, double *dw,
                                 double k1, double k2, cudaStream_t st) {
   using T = typename P::T;
   if (nbnd == 0) return cudaSuccess;
   const dim3 block(kBlockX);
-  const unsigned nb = static_cast<unsigned>(adr_list_blocks(nbnd));
+  const unsigned nb = static_cast<unsigned>((nbnd + kBlockX - 1) / kBlockX);
   const T *c = static_cast<const T *>(conc);
   switch (ns) {
     case 1: adj_grad_kernel<T, 1><<<nb, block, 0, st>>>(a, bnodes, nbnd, c, dkab, dkbc, fiber, dw, k1, k2); break;
