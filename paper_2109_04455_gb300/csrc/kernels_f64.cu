@@ -8,8 +8,7 @@ template cudaError_t launch_adr_flux<PrecF64>(int, const void *, const RefT *,
                                                  const uint32_t *, long long,
                                                  int, int, int, double *,
                                                  cudaStream_t);
-template cudaError_t launch_flow<PrecF64>(int, const FlowArgs &, dim3,
-                                             cudaStream_t);
+template cudaError_t launch_flow<PrecF64>(int, const FlowArgs &, cudaStream_t);
 template cudaError_t launch_adjoint<PrecF64>(int, int, const AdjArgs &,
                                                 cudaStream_t);
 template cudaError_t launch_adjoint_grad<PrecF64>(

@@ -45,13 +45,8 @@ inline long long plane_of(const lbm_geometry *g) {
   return static_cast<long long>(g->nx_pad) * g->ny;
 }
 
-inline dim3 lattice_grid(const lbm_geometry *g) {
-  return dim3(static_cast<unsigned>((g->nx_pad + kBlockX - 1) / kBlockX),
-              static_cast<unsigned>(g->ny));
-}
-
-inline long long grid_blocks(const lbm_geometry *g) {
-  const dim3 gr = lattice_grid(g);
+inline long long flow_blocks(const lbm_geometry *g) {
+  const dim3 gr = flow_grid(g->nx_pad, g->ny);
   return static_cast<long long>(gr.x) * gr.y;
 }
 
@@ -158,14 +153,14 @@ extern "C" size_t lbm_flow_ws_bytes(const lbm_geometry *g, int32_t precision) {
   const size_t p = static_cast<size_t>(plane_of(g));
   const size_t es = store_bytes(flow_prec(precision));
   return 2 * align256(9 * p * es) +
-         align256(static_cast<size_t>(grid_blocks(g)) * 2 * 8) +
+         align256(static_cast<size_t>(flow_blocks(g)) * 2 * 8) +
          align256(kReduceGrid * 2 * 8) + align256(64 * 8);
 }
 
-static cudaError_t flow_launch(int prec, int mode, const FlowArgs &a, dim3 grid,
+static cudaError_t flow_launch(int prec, int mode, const FlowArgs &a,
                                cudaStream_t st) {
-  return prec == LBM_F64 ? launch_flow<PrecF64>(mode, a, grid, st)
-                         : launch_flow<PrecF32>(mode, a, grid, st);
+  return prec == LBM_F64 ? launch_flow<PrecF64>(mode, a, st)
+                         : launch_flow<PrecF32>(mode, a, st);
 }
 
 extern "C" lbm_status lbm_flow_solve(const lbm_geometry *g,
@@ -203,12 +198,11 @@ extern "C" lbm_status lbm_flow_solve(const lbm_geometry *g,
   void *buf[2] = {b, b + bufb};
   double *partials = reinterpret_cast<double *>(b + 2 * bufb);
   double *scratch = reinterpret_cast<double *>(
-      b + 2 * bufb + align256(static_cast<size_t>(grid_blocks(g)) * 16));
+      b + 2 * bufb + align256(static_cast<size_t>(flow_blocks(g)) * 16));
   double *result = reinterpret_cast<double *>(
-      b + 2 * bufb + align256(static_cast<size_t>(grid_blocks(g)) * 16) +
+      b + 2 * bufb + align256(static_cast<size_t>(flow_blocks(g)) * 16) +
       align256(kReduceGrid * 2 * 8));
   cudaStream_t st = as_stream(stream);
-  const dim3 grid = lattice_grid(g);
 
   FlowArgs a{};
   a.links = g->d_links;
@@ -218,16 +212,31 @@ extern "C" lbm_status lbm_flow_solve(const lbm_geometry *g,
   a.nx = g->nx;
   a.ny = g->ny;
   a.nx_pad = g->nx_pad;
-  a.omega = 1.0 / p->tau;
+  // k1 = w_1 / tau with its last five bits cleared (Veltkamp's split), so that
+  // 3 k1 and 4.5 k1 are exact, and 1 - 1/tau less what that and the rounding
+  // took from the weights: the step then conserves mass and momentum as the
+  // scheme with the rounded weights does.  (With each constant rounded by
+  // itself the density drifts by up to 1e-16 per step.)
+  const double om = 1.0 / p->tau, w1 = 1.0 / 9.0;
+  const double c = 33.0 * (om * w1);
+  a.k1 = c - (c - om * w1);
+  a.keep = (1.0 - om) + 9.0 * std::fma(om, w1, -a.k1);
+  a.kh = 0.5 * a.keep;
+  a.k3 = 3.0 * a.k1;
+  a.k45 = 4.5 * a.k1;
   a.u0 = p->u0;
-  a.fomega = static_cast<float>(a.omega);
+  a.fkeep = static_cast<float>(a.keep);
+  a.fkh = static_cast<float>(a.kh);
+  a.fk1 = static_cast<float>(a.k1);
+  a.fk3 = static_cast<float>(a.k3);
+  a.fk45 = static_cast<float>(a.k45);
   a.fu0 = static_cast<float>(a.u0);
 
   cudaError_t e = cudaMemsetAsync(b, 0, 2 * bufb, st);
   if (e != cudaSuccess) return cuda_fail("lbm_flow_solve", e);
   a.src = nullptr;
   a.dst = buf[0];
-  e = flow_launch(prec, kFlowInit, a, grid, st);
+  e = flow_launch(prec, kFlowInit, a, st);
   if (e != cudaSuccess) return cuda_fail("lbm_flow_solve(init)", e);
   int cur = 0;
   int64_t steps = 0;
@@ -239,7 +248,7 @@ extern "C" lbm_status lbm_flow_solve(const lbm_geometry *g,
     a.dst = buf[cur ^ 1];
     cur ^= 1;
     ++steps;
-    return flow_launch(prec, mode, a, grid, st);
+    return flow_launch(prec, mode, a, st);
   };
   // n steps, the last two writing u and the residual sums
   auto chunk = [&](int64_t n) -> lbm_status {
@@ -250,7 +259,7 @@ extern "C" lbm_status lbm_flow_solve(const lbm_geometry *g,
     cudaError_t e2 = step(kFlowU);
     if (e2 == cudaSuccess) e2 = step(kFlowCheck);
     if (e2 == cudaSuccess)
-      e2 = launch_reduce(2, 0, partials, grid_blocks(g), scratch, result, st);
+      e2 = launch_reduce(2, 0, partials, flow_blocks(g), scratch, result, st);
     double h[2] = {0, 0};
     if (e2 == cudaSuccess)
       e2 = cudaMemcpyAsync(h, result, sizeof(h), cudaMemcpyDeviceToHost, st);

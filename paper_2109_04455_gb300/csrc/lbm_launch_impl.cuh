@@ -66,18 +66,23 @@ cudaError_t launch_adr_flux(int ns, const void *g, const RefT *ref,
   return cudaGetLastError();
 }
 
-template <class P>
-cudaError_t launch_flow(int mode, const FlowArgs &a, dim3 grid,
-                        cudaStream_t st) {
-  const dim3 block(kBlockX);
+template <class P, int BX>
+static cudaError_t launch_flow_bx(int mode, const FlowArgs &a, cudaStream_t st) {
+  const dim3 grid = flow_grid(a.nx_pad, a.ny);
   switch (mode) {
-    case kFlowStep: flow_kernel<P, kFlowStep><<<grid, block, 0, st>>>(a); break;
-    case kFlowU: flow_kernel<P, kFlowU><<<grid, block, 0, st>>>(a); break;
-    case kFlowCheck: flow_kernel<P, kFlowCheck><<<grid, block, 0, st>>>(a); break;
-    case kFlowInit: flow_kernel<P, kFlowInit><<<grid, block, 0, st>>>(a); break;
+    case kFlowStep: flow_kernel<P, kFlowStep, BX><<<grid, BX, 0, st>>>(a); break;
+    case kFlowU: flow_kernel<P, kFlowU, BX><<<grid, BX, 0, st>>>(a); break;
+    case kFlowCheck: flow_kernel<P, kFlowCheck, BX><<<grid, BX, 0, st>>>(a); break;
+    case kFlowInit: flow_kernel<P, kFlowInit, BX><<<grid, BX, 0, st>>>(a); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
+}
+
+template <class P>
+cudaError_t launch_flow(int mode, const FlowArgs &a, cudaStream_t st) {
+  return flow_block_x(a.nx_pad, a.ny) == 64 ? launch_flow_bx<P, 64>(mode, a, st)
+                                            : launch_flow_bx<P, 256>(mode, a, st);
 }
 
 template <class P>

@@ -73,3 +73,20 @@ def test_adr_step_shapes(shape, ns):
                        rtol=1e-12, atol=0)
     assert np.allclose(info["flux"][:ns], ref["flux"][:ns], rtol=1e-10,
                        atol=1e-15)
+
+
+@pytest.mark.parametrize("shape", SHAPES)
+def test_flow_step_shapes(shape):
+    nx, ny = shape
+    fib = _fibers(nx, ny)
+    solid, _, _ = oracle.raster(nx, ny, fib, 0.0, 0.0)
+    geom = lbm.Geometry(nx, ny, fib, 0.0, 0.0).upload()
+    u, info = lbm.lbm_flow_solve(geom, 0.7, 0.05, STEPS,
+                                 precision=lbm.LBM_F64)
+    _, ux, uy, res = oracle.flow_run(solid, 0.7, 0.05, STEPS)
+    got = u.cpu().numpy()[:, :, :nx]
+    # velocities are differences of populations of order one: 40 steps of
+    # about 20 roundings of 1.1e-16 stay below 1e-13
+    assert np.abs(got[0] - ux).max() < 1e-13
+    assert np.abs(got[1] - uy).max() < 1e-13
+    assert info["residual"] == pytest.approx(res, rel=1e-8)
