@@ -216,7 +216,8 @@ def _peak_hbm():
 
 
 KERNEL_SOURCES = {
-    "f32": ("lbm_kernels.cuh", "lbm_launch_impl.cuh", "kernels_f32.cu"),
+    "f32": ("lbm_kernels.cuh", "lbm_twostep.cuh", "lbm_launch_impl.cuh",
+            "kernels_f32.cu"),
     "f16dev": ("lbm_kernels.cuh", "lbm_launch_impl.cuh", "lbm_f16.cuh",
                "kernels_f16dev.cu"),
     "f64": ("lbm_kernels.cuh", "lbm_launch_impl.cuh", "kernels_f64.cu"),
@@ -255,8 +256,14 @@ def _ncu_traffic(precision: str, units_per_launch: int):
         return None
 
 
+def _steps_per_launch(geom, precision):
+    """Plain steps per launch (and per pass over memory): FP32 lattices of
+    2^22 nodes or more take two."""
+    return 2 if precision == "f32" and geom.nx_pad * geom.ny >= 1 << 22 else 1
+
+
 def _algorithmic_bytes(geom, w, precision):
-    """Bytes one ADR step must move: per fluid node 3 species x 9
+    """Bytes one launch of the ADR step must move: per fluid node 3 species x 9
     populations read + written, the velocity (2 values) and the link word
     (half storage: also each species' half reference, read + written; FP64:
     the nine equilibrium factors instead of the velocity); per solid node
@@ -437,22 +444,21 @@ def _measure(precision, geom, w, u, steps, warmup, dev, world, fp64_peak):
         dist.barrier()
     elapsed = max_over_ranks(t0.elapsed_time(t1) * 1e-3, dev)
     plain_s = sum(e0.elapsed_time(e1) for e0, e1 in ev_plain) * 1e-3
-    # per ADR step the bulk kernel and (when the lattice has boundary nodes)
-    # the boundary-node kernel; per bench step the two-level partial-sum
-    # reduce (2 launches) and the outflux kernel
-    lw = geom.ws[:4 * geom.nx_pad * geom.ny].view(torch.int32).cpu().numpy()
-    has_bnd = bool(((lw != 0) & (lw != -1)).any())
-    launches_per_step = CHUNK * (2 if has_bnd else 1) + 3
+    # per bench step the plain steps' launches, the two check steps, the
+    # two-level partial-sum reduce (2 launches) and the outflux kernel
+    per_launch = _steps_per_launch(geom, precision)
+    launches_per_step = (CHUNK - 2) // per_launch + 2 + 3
     updates = SPECIES * w.nx * w.ny * CHUNK * steps
     value = job_throughput(updates, world, elapsed)
     alg_bytes, n_fluid, per_fluid = _algorithmic_bytes(geom, w, precision)
-    step_launch_s = plain_s / ((CHUNK - 2) * steps)
+    step_launch_s = plain_s / ((CHUNK - 2) * steps) * per_launch
     achieved = alg_bytes / step_launch_s / 1e9
     peak, peak_kind = _peak_hbm()
     traffic = _ncu_traffic(precision, n_fluid)
-    kernel = ("adr_bulk_quad_kernel<3 species> (f16dev, plain steps)"
+    kernel = ("adr_step_quad_kernel<3 species> (f16dev, plain steps)"
               if precision == "f16dev" else
-              f"adr_bulk_kernel<{precision},3 species,step>")
+              "adr_two_step_kernel<3 species>" if per_launch == 2 else
+              f"adr_step_kernel<{precision},3 species,step>")
     if precision != "f64":
         roof = {"bound": "hbm", "achieved": achieved, "peak": peak,
                 "unit": "GB/s", "frac": achieved / peak,
@@ -467,7 +473,8 @@ def _measure(precision, geom, w, u, steps, warmup, dev, world, fp64_peak):
     roof.update({"traffic": traffic, "kernel": kernel,
                  "algorithmic_bytes_per_launch": alg_bytes,
                  "bytes_per_fluid_node": per_fluid, "fluid_nodes": n_fluid,
-                 "avg_launch_ms": step_launch_s * 1e3})
+                 "avg_launch_ms": step_launch_s * 1e3,
+                 "steps_per_launch": per_launch})
     rec = {"value": value, "unit": UNIT, "steps": steps, "warmup": warmup,
            "ms_per_step": elapsed / steps * 1e3,
            "dtype": {"f32": "f32", "f16dev": "f16-storage/f32-compute",

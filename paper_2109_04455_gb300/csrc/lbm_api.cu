@@ -469,6 +469,7 @@ extern "C" lbm_status lbm_adr_create(const lbm_geometry *g,
   a.nx_pad = g->nx_pad;
   a.abb_all = (p->flags & LBM_ADR_INLET_ABB_ALL) ? 1 : 0;
   a.nodewise = (p->flags & LBM_ADR_NODEWISE) ? 1 : 0;
+  a.periodic = g->periodic;
   for (int k = 0; k < 3; ++k) {
     const bool on = k < p->nspecies;
     a.omega[k] = on ? 1.0 / p->tau[k] : 0.0;
@@ -511,7 +512,8 @@ extern "C" lbm_status lbm_adr_init(lbm_adr_solver *s, void *stream) {
   return LBM_OK;
 }
 
-static cudaError_t adr_step(lbm_adr_solver *s, int mode, cudaStream_t st) {
+// arguments of the launch that takes the state from one buffer to the other
+static AdrArgs adr_next(lbm_adr_solver *s, int steps) {
   AdrArgs a = s->a;
   a.src = s->buf[s->cur];
   a.dst = s->buf[s->cur ^ 1];
@@ -519,8 +521,28 @@ static cudaError_t adr_step(lbm_adr_solver *s, int mode, cudaStream_t st) {
   a.rdst = s->rbuf[s->cur ^ 1];
   a.step = static_cast<unsigned>(s->steps);
   s->cur ^= 1;
-  ++s->steps;
-  return adr_launch(s->p.precision, s->p.nspecies, mode, a, st);
+  s->steps += steps;
+  return a;
+}
+
+static cudaError_t adr_step(lbm_adr_solver *s, int mode, cudaStream_t st) {
+  return adr_launch(s->p.precision, s->p.nspecies, mode, adr_next(s, 1), st);
+}
+
+// n plain steps
+static cudaError_t adr_plain_steps(lbm_adr_solver *s, int64_t n, cudaStream_t st) {
+  cudaError_t e = cudaSuccess;
+  const bool two = two_step_pays(s->p.precision, s->p.nspecies, s->a.plane);
+  for (int64_t k = 0; k < n && e == cudaSuccess;) {
+    if (two && n - k >= 2) {
+      e = launch_adr_two_step(s->p.nspecies, adr_next(s, 2), st);
+      k += 2;
+    } else {
+      e = adr_step(s, kAdrStep, st);
+      k += 1;
+    }
+  }
+  return e;
 }
 
 extern "C" lbm_status lbm_adr_run(lbm_adr_solver *s, int64_t nsteps,
@@ -534,12 +556,10 @@ extern "C" lbm_status lbm_adr_run(lbm_adr_solver *s, int64_t nsteps,
   cudaStream_t st = as_stream(stream);
   const int ns = s->p.nspecies;
   const int64_t plain = info ? nsteps - 2 : nsteps;
-  for (int64_t k = 0; k < plain; ++k) {
-    cudaError_t e = adr_step(s, kAdrStep, st);
-    if (e != cudaSuccess) return cuda_fail("lbm_adr_run(step)", e);
-  }
+  cudaError_t e = adr_plain_steps(s, plain, st);
+  if (e != cudaSuccess) return cuda_fail("lbm_adr_run(step)", e);
   if (!info) return LBM_OK;
-  cudaError_t e = adr_step(s, kAdrCheck, st);
+  e = adr_step(s, kAdrCheck, st);
   if (e == cudaSuccess) e = adr_step(s, kAdrCheck, st);
   if (e == cudaSuccess)
     e = launch_reduce(2 * ns, ns, s->partials, s->nb, s->scratch, s->result, st);

@@ -268,6 +268,7 @@ struct AdrArgs {
                             // beyond them takes boundary-node chunks
   int abb_all;              // anti-bounce-back inlet for every species
   int nodewise;             // every population of a reactive node reacts
+  int periodic;             // LBM_PERIODIC_X | LBM_PERIODIC_Y
   unsigned step;            // steps done before this one (rounding seed)
   int xp;                   // flux plane
   double omega[3];          // 1/tau per species
@@ -411,72 +412,112 @@ __device__ __forceinline__ void add_source(const AdrArgs &a, int s, uint32_t lw,
   }
 }
 
-// Update of a boundary node (x, y) (a fluid node with link word lw != 0): the
-// pulls, with the rule of the link's type wherever the source x - c_i is not
-// a fluid node (Eq. BC and bounce-back: all of them read the node's own
-// opposite population), BGK towards C E_i, then the Dawson source on links
-// into catalytic fiber nodes (Eq. source_lbm), or, with a.nodewise, on all
-// nine populations with the mean rates of those links.  put(s, g, c) stores
-// the new populations of species s.
+// The old populations that the update of node (link word lw) reads, into g:
+// the pulls from x - c_i, or, where the source is not a fluid node, the
+// node's own opposite population, to which update_node then applies the rule
+// of the link's type (Eq. BC and bounce-back).
 //
-// The node's latency bounds the step of a small lattice (a 200 x 100 one took
-// 23 us per step with each load behind its link's branch, species after
-// species), so every load is issued before any arithmetic: there is exactly
-// one per population, whatever the link types, from a selected place.
-template <int NS, class Src, typename T, class Put>
-__device__ __forceinline__ void boundary_update(const AdrArgs &a, const Src &src,
-                                                uint32_t lw, int x, int y,
-                                                const T (&E)[9], Put &&put) {
-  T g[NS][9], cb[NS], ka[9], kb[9];
-  bool outlet = false, cat = false;
+// There is one load per population whatever the link types, from a selected
+// place, and all are issued before any arithmetic: the boundary nodes'
+// latency bounds the step of a small lattice (a 200 x 100 one took 23 us per
+// step with each load behind its link's branch, species after species).
+template <int NS, class Src, typename T>
+__device__ __forceinline__ void gather_node(const Src &src, uint32_t lw, T (&g)[NS][9]) {
+  if (lw == 0u) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const auto from = src.at(i, opp(i), kFluid);
+#pragma unroll
+      for (int s = 0; s < NS; ++s) g[s][i] = src.get(s, from);
+    }
+    return;
+  }
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
     const uint32_t t = i == 0 ? (uint32_t)kFluid : nib(lw, opp(i));
     const bool pulled = t == kFluid || t == kPeriodic;
-    outlet = outlet || t == kOutlet;
-    cat = cat || t == kCat;
     const auto from = pulled ? src.at(i, opp(i), t) : src.at(opp(i), 0, kFluid);
 #pragma unroll
     for (int s = 0; s < NS; ++s) g[s][i] = src.get(s, from);
   }
-  if (cat) {
-    const long long np = a.nx_pad;
+}
+
+// The inlet and outlet rules of a node of the first or last column (link
+// word lw), species s: g holds the node's own opposite populations there.
+// cb: the node's own concentration (outlet).
+template <typename T>
+__device__ __forceinline__ void edge_rules(const AdrArgs &a, int s, uint32_t lw,
+                                           T cb, T (&g)[9]) {
+#pragma unroll
+  for (int i = 1; i < 9; ++i) {
+    const uint32_t t = nib(lw, opp(i));
+    const T w2 = T(2) * Lattice<T>::w(i);
+    if (t == kInlet && (s == 0 || a.abb_all))
+      g[i] = fma_rn(w2, pick<T>(a.cin[s], a.fcin[s]), -g[i]);
+    else if (t == kOutlet)
+      g[i] = fma_rn(w2, cb, -g[i]);
+  }
+}
+
+// BGK of species s towards C E_i; returns C.
+template <typename T>
+__device__ __forceinline__ T collide(const AdrArgs &a, int s, const T (&E)[9], T (&g)[9]) {
+  const T c = sum_rn(g), om = pick<T>(a.omega[s], a.fomega[s]);
+#pragma unroll
+  for (int i = 0; i < 9; ++i) g[i] = relax(om, c, E[i], g[i]);
+  return c;
+}
+
+// Update of node (x, y) from its gathered populations g: the rules of its
+// links, BGK towards C E_i, then the Dawson source on links into catalytic
+// fiber nodes (Eq. source_lbm), or, with a.nodewise, on all nine populations
+// with the mean rates of those links.  put(s, g, c) stores the new
+// populations of species s, whose concentration is c.
+template <int NS, class Src, typename T, class Put>
+__device__ __forceinline__ void update_node(const AdrArgs &a, const Src &src,
+                                            uint32_t lw, int x, int y,
+                                            const T (&E)[9], T (&g)[NS][9],
+                                            Put &&put) {
+  T ka[9], kb[9];
+  bool cat = false;
+  if (lw != 0u) {
+    bool inlet = false, outlet = false;
 #pragma unroll
     for (int j = 1; j < 9; ++j) {
-      const bool on = nib(lw, j) == kCat;
-      const long long m = on ? neighbour(x, y, j, a.nx, a.ny, np) : 0;
-      ka[j] = on ? T(a.kab[m]) : T(0);
-      kb[j] = on ? T(a.kbc[m]) : T(0);
+      const uint32_t t = nib(lw, j);
+      inlet = inlet || t == kInlet;
+      outlet = outlet || t == kOutlet;
+      cat = cat || t == kCat;
     }
-  }
-  if (outlet) {   // C_w = the node's own concentration
+    if (cat) {
 #pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      T own[9];
+      for (int j = 1; j < 9; ++j) {
+        const bool on = nib(lw, j) == kCat;
+        const long long m = on ? neighbour(x, y, j, a.nx, a.ny, a.nx_pad) : 0;
+        ka[j] = on ? T(a.kab[m]) : T(0);
+        kb[j] = on ? T(a.kbc[m]) : T(0);
+      }
+    }
+    if (inlet || outlet) {
 #pragma unroll
-      for (int j = 0; j < 9; ++j) own[j] = src.get(s, src.at(j, 0, kFluid));
-      cb[s] = sum_rn(own);
+      for (int s = 0; s < NS; ++s) {
+        T cb = T(0);
+        if (outlet) {   // C_w = the node's own concentration
+          T own[9];
+#pragma unroll
+          for (int j = 0; j < 9; ++j) own[j] = src.get(s, src.at(j, 0, kFluid));
+          cb = sum_rn(own);
+        }
+        edge_rules(a, s, lw, cb, g[s]);
+      }
     }
   }
   T C[NS];
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
-#pragma unroll
-    for (int i = 1; i < 9; ++i) {
-      const uint32_t t = nib(lw, opp(i));
-      const T w2 = T(2) * Lattice<T>::w(i);
-      if (t == kInlet && (s == 0 || a.abb_all))
-        g[s][i] = fma_rn(w2, pick<T>(a.cin[s], a.fcin[s]), -g[s][i]);
-      else if (t == kOutlet)
-        g[s][i] = fma_rn(w2, cb[s], -g[s][i]);
-    }
-    const T c = sum_rn(g[s]);
-    C[s] = c;
-    const T om = pick<T>(a.omega[s], a.fomega[s]);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) g[s][i] = relax(om, c, E[i], g[s][i]);
+    C[s] = collide(a, s, E, g[s]);
     if (cat) add_source<NS>(a, s, lw, ka, kb, C, g[s]);
-    put(s, g[s], c);
+    put(s, g[s], C[s]);
   }
 }
 
@@ -512,10 +553,11 @@ __device__ __forceinline__ void adr_boundary_node(const AdrArgs &a, long long n,
 #pragma unroll
     for (int s = 0; s < NS; ++s) prev[s] = cp[s * a.plane + n];
   }
-  T E[9];
+  const GlobalSource<P> src{a, n, x, y};
+  T g[NS][9], E[9];
+  gather_node<NS>(src, lw, g);
   adr_eq<P>(a, n, E);
-  boundary_update<NS>(a, GlobalSource<P>{a, n, x, y}, lw, x, y, E,
-                      [&](int s, const T (&g)[9], T c) {
+  update_node<NS>(a, src, lw, x, y, E, g, [&](int s, const T (&g)[9], T c) {
     put_node<P>(a, s, n, g, c);
     if (MODE == kAdrCheck) {
       check_add<NS, T>(acc, s, c, prev[s]);
@@ -718,6 +760,11 @@ __global__ void __launch_bounds__(BX, BX == 256 ? P::kMinBlocks : 1)
       block_partials_store<2 * NS, NS, 1, BX, T>(acc, a.partials + row * (3 * NS));
   }
 }
+
+}  // namespace lbm
+// two FP32 steps in one pass over memory
+#include "lbm_twostep.cuh"
+namespace lbm {
 
 // Outflux on the plane x = xp from the stored post-collision populations:
 // out[s] = (1/ny) sum_y sum_i c_ix g*_{s,i}(xp, y).  One block.
@@ -1016,6 +1063,9 @@ inline long long adr_partial_rows(int prec, int nx_pad, int ny, long long nbnd) 
 
 template <class P>
 cudaError_t launch_adr(int ns, int mode, const AdrArgs &a, cudaStream_t st);
+// two plain steps in one launch (FP32), and whether they are worth it
+bool two_step_pays(int prec, int ns, long long plane);
+cudaError_t launch_adr_two_step(int ns, const AdrArgs &a, cudaStream_t st);
 template <class P>
 cudaError_t launch_adr_flux(int ns, const void *g, const RefT *ref,
                             const uint32_t *links, long long plane, int nx_pad,
