@@ -450,9 +450,9 @@ lbm_status lbm_rwpt_run(lbm_rwpt *r, int64_t nsteps, void *stream,
 /* Zero the outlet counts and start a new window. */
 lbm_status lbm_rwpt_reset_counts(lbm_rwpt *r, void *stream);
 
-/* Copy the particles (in storage order, which varies from run to run) to
- * host arrays of max_count entries; *count receives their number
- * (LBM_ENOMEM if it exceeds max_count). */
+/* Copy the particles, in the order of their ids, to host arrays of max_count
+ * entries; *count receives their number (LBM_ENOMEM if it exceeds
+ * max_count). */
 lbm_status lbm_rwpt_particles(lbm_rwpt *r, void *stream, int64_t max_count,
                               int64_t *count, double *x, double *y,
                               int32_t *species, uint64_t *id);

@@ -628,8 +628,7 @@ class RWPT:
             x.ctypes.data_as(_P), y.ctypes.data_as(_P), s.ctypes.data_as(_P),
             ids.ctypes.data_as(_P)))
         m = cnt.value
-        o = np.argsort(ids[:m], kind="stable")
-        return x[:m][o], y[:m][o], s[:m][o], ids[:m][o]
+        return x[:m].copy(), y[:m].copy(), s[:m].copy(), ids[:m].copy()
 
     def close(self):
         if self.handle:
