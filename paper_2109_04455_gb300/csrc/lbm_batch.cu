@@ -3,14 +3,15 @@
 // between convergence checks; the launch shape is picked by a small
 // autotuner that times the candidates on the batch itself.
 //
-// Work list: every active instance contributes its interior row tiles (BX
-// consecutive nodes of one row) and its boundary-node chunks (BX entries of
-// its boundary list).  Items are stored instance by instance, so each
+// Work list: every active instance contributes its interior row tiles (TILE
+// consecutive nodes of one row) and its boundary-node chunks (chunk_len
+// entries of its boundary list).  Items are stored instance by instance, so each
 // instance's check-step partial sums occupy a contiguous row range.  A
 // persistent grid of blocks walks the list; per item the instance's
 // arguments are staged in shared memory and the same per-node updates as the
-// single-lattice kernels run (adr_interior_node / adr_boundary_node), so a
-// batched solve gives the same populations as lbm_adr_solve on each lattice.
+// single-lattice kernels run (adr_interior_node, quad_segment, pair_segment
+// and adr_boundary_node), so a batched solve gives the same populations as
+// lbm_adr_solve on each lattice.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -41,16 +42,33 @@ __host__ __device__ inline unsigned long long chunk_item(int inst,
          static_cast<unsigned long long>(start);
 }
 
+// Threads of a step's block: one node each, or with half storage four (plain
+// step) or two (check step) of a tile's nodes.  With one node per thread the
+// half batch took as long as the FP32 one: 390 us per step of 16 lattices, 7.9
+// million nodes, against 273 us with four (and 168 registers: at 128 they
+// spill, 286 us).
+template <class P, int MODE, int TILE>
+struct StepThreads {
+  static constexpr int value = !P::kDev ? TILE : MODE == kAdrCheck ? TILE / 2 : TILE / 4;
+};
+// entries of a boundary chunk: no more than either step's threads
+inline long long chunk_len(int prec, int tile) {
+  return prec == LBM_F16DEV ? tile / 4 : tile;
+}
+
 // stepc[parity]: steps every active instance has done before this one (all
 // start together); the launch passes it to the per-node updates as
 // AdrArgs::step (the rounding seed of half storage) and leaves the next
 // count in stepc[parity ^ 1] for the next launch.
-template <class P, int NS, int MODE, int BX>
-__global__ void __launch_bounds__(BX)
+template <class P, int NS, int MODE, int TILE>
+__global__ void __launch_bounds__(StepThreads<P, MODE, TILE>::value,
+                                  !P::kDev ? 1 : MODE == kAdrCheck ? 1024 / TILE : 1536 / TILE)
     batch_step_kernel(const AdrArgs *__restrict__ table, int parity,
                       const unsigned long long *__restrict__ work,
                       long long nwork, double *partials, unsigned *stepc) {
   using T = typename P::T;
+  constexpr int BX = StepThreads<P, MODE, TILE>::value;
+  constexpr int kPer = P::kDev && MODE == kAdrCheck ? 2 : 1;   // partial values a thread
   __shared__ AdrArgs sa;
   constexpr int kWords = sizeof(AdrArgs) / sizeof(unsigned long long);
   static_assert(sizeof(AdrArgs) % sizeof(unsigned long long) == 0,
@@ -59,11 +77,19 @@ __global__ void __launch_bounds__(BX)
   constexpr int kStepShift = static_cast<int>(offsetof(AdrArgs, step) % 8) * 8;
   const unsigned step = stepc[parity];
   if (blockIdx.x == 0 && threadIdx.x == 0) stepc[parity ^ 1] = step + 1u;
+  // the next item's word is on its way while this one is worked on, and the
+  // arguments are staged only when the instance changes
+  unsigned long long following = blockIdx.x < nwork ? work[blockIdx.x] : 0ull;
+  int staged = -1;
   for (long long w = blockIdx.x; w < nwork; w += gridDim.x) {
-    const unsigned long long item = work[w];
+    const unsigned long long item = following;
+    if (w + gridDim.x < nwork) following = work[w + gridDim.x];
     const int inst = static_cast<int>((item >> 48) & 0x7fff);
-    __syncthreads();  // the previous item is done with sa
-    {
+    // the previous item is done with sa (and, on check steps, with the
+    // partial sums' shared memory)
+    if (MODE == kAdrCheck || inst != staged) __syncthreads();
+    if (inst != staged) {
+      staged = inst;
       const unsigned long long *srcw =
           reinterpret_cast<const unsigned long long *>(table + 2 * inst + parity);
       unsigned long long *dstw = reinterpret_cast<unsigned long long *>(&sa);
@@ -74,28 +100,37 @@ __global__ void __launch_bounds__(BX)
               (static_cast<unsigned long long>(step) << kStepShift);
         dstw[k] = v;
       }
+      __syncthreads();
     }
-    __syncthreads();
-    T acc[1][3 * NS];
+    T acc[kPer][3 * NS];
 #pragma unroll
-    for (int k = 0; k < 3 * NS; ++k) acc[0][k] = T(0);
+    for (int p = 0; p < kPer; ++p)
+#pragma unroll
+      for (int k = 0; k < 3 * NS; ++k) acc[p][k] = T(0);
     if (!(item & kChunkBit)) {
-      const long long y = static_cast<long long>((item >> 24) & 0xffffff);
-      const long long xb = static_cast<long long>(item & 0xffffff);
-      const int x = static_cast<int>(xb * BX + threadIdx.x);
-      const long long n = y * sa.nx_pad + x;
-      const uint32_t lw = (x < sa.nx_pad) ? sa.links[n] : kSolidNode;
-      if (lw == 0u) adr_interior_node<P, NS, MODE>(sa, n, acc[0]);
+      const int y = static_cast<int>((item >> 24) & 0xffffff);
+      const int x0 = static_cast<int>(item & 0xffffff) * TILE;
+      if constexpr (P::kDev) {
+        if constexpr (MODE == kAdrCheck)
+          pair_segment<NS, MODE, BX>(sa, y, x0, acc);
+        else
+          quad_segment<NS, BX>(sa, y, x0);
+      } else {
+        const int x = x0 + threadIdx.x;
+        const long long n = (long long)y * sa.nx_pad + x;
+        const uint32_t lw = (x < sa.nx_pad) ? sa.links[n] : kSolidNode;
+        if (lw == 0u) adr_interior_node<P, NS, MODE>(sa, n, acc[0]);
+      }
     } else {
       const long long t =
           static_cast<long long>(item & ((1ull << 48) - 1)) + threadIdx.x;
-      if (t < sa.nbnd) {
+      if (t < sa.nbnd && (!P::kDev || threadIdx.x < TILE / 4)) {
         const BoundaryNode b = sa.bnodes[t];
         adr_boundary_node<P, NS, MODE>(sa, b.n, b.links, acc[0]);
       }
     }
     if constexpr (MODE == kAdrCheck)
-      block_partials_store<2 * NS, NS, 1, BX, T>(acc, partials + w * (3 * NS));
+      block_partials_store<2 * NS, NS, kPer, BX, T>(acc, partials + w * (3 * NS));
   }
 }
 
@@ -153,23 +188,26 @@ __global__ void __launch_bounds__(kReduceThreads)
   block_sum_store<NS, double>(acc, out + (long long)blockIdx.x * 3);
 }
 
+template <class P, int NS, int MODE, int TILE>
+cudaError_t launch_step_t(const AdrArgs *table, int parity,
+                          const unsigned long long *work, long long nwork,
+                          double *partials, unsigned *stepc, unsigned grid,
+                          cudaStream_t st) {
+  batch_step_kernel<P, NS, MODE, TILE><<<grid, StepThreads<P, MODE, TILE>::value, 0, st>>>(
+      table, parity, work, nwork, partials, stepc);
+  return cudaGetLastError();
+}
+
 template <class P, int NS>
 cudaError_t launch_step(int mode, int bx, const AdrArgs *table, int parity,
                         const unsigned long long *work, long long nwork,
                         double *partials, unsigned *stepc, unsigned grid,
                         cudaStream_t st) {
-  if (bx == 128) {
-    if (mode == kAdrCheck)
-      batch_step_kernel<P, NS, kAdrCheck, 128><<<grid, 128, 0, st>>>(table, parity, work, nwork, partials, stepc);
-    else
-      batch_step_kernel<P, NS, kAdrStep, 128><<<grid, 128, 0, st>>>(table, parity, work, nwork, partials, stepc);
-  } else {
-    if (mode == kAdrCheck)
-      batch_step_kernel<P, NS, kAdrCheck, 256><<<grid, 256, 0, st>>>(table, parity, work, nwork, partials, stepc);
-    else
-      batch_step_kernel<P, NS, kAdrStep, 256><<<grid, 256, 0, st>>>(table, parity, work, nwork, partials, stepc);
-  }
-  return cudaGetLastError();
+  const auto f = bx == 128 ? (mode == kAdrCheck ? launch_step_t<P, NS, kAdrCheck, 128>
+                                                : launch_step_t<P, NS, kAdrStep, 128>)
+                           : (mode == kAdrCheck ? launch_step_t<P, NS, kAdrCheck, 256>
+                                                : launch_step_t<P, NS, kAdrStep, 256>);
+  return f(table, parity, work, nwork, partials, stepc, grid, st);
 }
 
 template <class P>
@@ -193,18 +231,18 @@ cudaError_t launch_flux_p(int ns, int count, const AdrArgs *table, int parity,
   return cudaGetLastError();
 }
 
+template <class P, int TILE>
+int occupancy_t(int ns) {
+  int nb = 0;
+  constexpr int kThreads = StepThreads<P, kAdrStep, TILE>::value;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+      &nb, ns == 2 ? batch_step_kernel<P, 2, kAdrStep, TILE>
+                   : batch_step_kernel<P, 3, kAdrStep, TILE>, kThreads, 0);
+  return nb > 0 ? nb : 1;
+}
 template <class P>
 int occupancy(int ns, int bx) {
-  int nb = 0;
-  if (bx == 128)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &nb, ns == 2 ? batch_step_kernel<P, 2, kAdrStep, 128>
-                     : batch_step_kernel<P, 3, kAdrStep, 128>, 128, 0);
-  else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &nb, ns == 2 ? batch_step_kernel<P, 2, kAdrStep, 256>
-                     : batch_step_kernel<P, 3, kAdrStep, 256>, 256, 0);
-  return nb > 0 ? nb : 1;
+  return bx == 128 ? occupancy_t<P, 128>(ns) : occupancy_t<P, 256>(ns);
 }
 
 inline size_t a256(size_t n) { return (n + 255) / 256 * 256; }
@@ -259,10 +297,11 @@ lbm_status bfail(const char *where, cudaError_t e) {
   return LBM_ECUDA;
 }
 
-long long items_of(const lbm_geometry *g, int bx) {
+long long items_of(const lbm_geometry *g, int prec, int bx) {
   const long long tiles = static_cast<long long>((g->nx_pad + bx - 1) / bx) * g->ny;
   const long long nb = static_cast<long long>(g->bnodes.size());
-  return tiles + (nb + bx - 1) / bx;
+  const long long len = chunk_len(prec, bx);
+  return tiles + (nb + len - 1) / len;
 }
 
 size_t store_b(int prec) { return prec == LBM_F64 ? 8 : (prec == LBM_F32 ? 4 : 2); }
@@ -281,7 +320,7 @@ BatchLayout batch_layout(int count, const lbm_geometry *const *geoms,
   BatchLayout l{};
   const int ns = p[0].nspecies;
   long long items = 0;
-  for (int i = 0; i < count; ++i) items += items_of(geoms[i], 128);
+  for (int i = 0; i < count; ++i) items += items_of(geoms[i], p[0].precision, 128);
   l.table = a256(sizeof(AdrArgs) * 2 * count);
   l.work = a256(8 * items);
   l.partials = a256(8 * 3 * ns * items);
@@ -373,7 +412,8 @@ cudaError_t build_work(lbm_batch *b, cudaStream_t st) {
       for (long long y = 0; y < g->ny; ++y)
         for (long long xb = 0; xb < nxb; ++xb) b->work.push_back(tile_item(i, y, xb));
       const long long nb = static_cast<long long>(g->bnodes.size());
-      for (long long t = 0; t < nb; t += b->bx) b->work.push_back(chunk_item(i, t));
+      for (long long t = 0; t < nb; t += chunk_len(b->prec, b->bx))
+        b->work.push_back(chunk_item(i, t));
     }
     b->rows[2 * i] = lo;
     b->rows[2 * i + 1] = static_cast<long long>(b->work.size());

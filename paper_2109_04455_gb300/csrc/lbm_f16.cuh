@@ -1,7 +1,6 @@
 // FP16-deviation storage (populations stored as half of 2^14 (g - w_i R),
 // R the storing node's concentration, itself stored in half): the update of
-// an interior node, in a one-node form (used by the batch kernel) and a
-// two-node bulk kernel.  Included by lbm_kernels.cuh after AdrArgs and the
+// interior nodes, four per thread (plain steps) and two (check steps).  Included by lbm_kernels.cuh after AdrArgs and the
 // lattice helpers.
 #pragma once
 
@@ -14,66 +13,23 @@ namespace lbm {
 // is brought back to scale 1 once per species and node.  Scaling by a power
 // of two is exact, so every result equals the unscaled arithmetic's.  Each
 // operation is written with an explicit rounding (no contraction left to
-// the compiler), so the one-node form (batch kernel) and the two-node form
-// (bulk step) give the same bits for the same node.
+// the compiler), so both forms give the same bits for the same node.
 // ---------------------------------------------------------------------------
 namespace f16 {
 constexpr float kDown = 1.0f / 16384.0f, kUp = 16384.0f;
 __device__ __forceinline__ float w(int i) { return Lattice<float>::w(i); }
-// scaled population pulled from a source node: its stored deviation h plus
-// w_i 2^14 times the source's reference concentration r (as stored, at
-// scale 1).  w_i 2^14 is exact, so this equals fma(w_i, 2^14 r, h) bit for
-// bit, without the multiply by 2^14.
-__device__ __forceinline__ float pull(int i, float h, float r) {
-  return __fmaf_rn(w(i) * kUp, r, h);
-}
-// equilibrium factors E_i(u) = w_i (1 + 3 c.u + 4.5 (c.u)^2 - 1.5 u.u),
-// built for each direction together with its opposite (c.u changes sign,
-// the even part w_i (1 + 4.5 (c.u)^2 - 1.5 u.u) is shared)
-__device__ __forceinline__ void eq(float ux, float uy, float (&E)[9]) {
-  const float base = __fmaf_rn(-1.5f, __fmaf_rn(ux, ux, __fmul_rn(uy, uy)), 1.0f);
-  E[0] = __fmul_rn(w(0), base);
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int i = k < 2 ? k + 1 : k + 3;   // 1, 2, 5, 6
-    const float cu = __fadd_rn(float(cx(i)) * ux, float(cy(i)) * uy);
-    const float even = __fmul_rn(w(i), __fmaf_rn(__fmul_rn(4.5f, cu), cu, base));
-    E[i] = __fmaf_rn(3.0f * w(i), cu, even);
-    E[opp(i)] = __fmaf_rn(-3.0f * w(i), cu, even);
-  }
-}
-// C_s at scale 2^14: a pairwise sum (short dependency chains)
-__device__ __forceinline__ float sum9(const float (&g)[9]) {
-  const float a = __fadd_rn(__fadd_rn(g[0], g[1]), __fadd_rn(g[2], g[3]));
-  const float b = __fadd_rn(__fadd_rn(g[4], g[5]), __fadd_rn(g[6], g[7]));
-  return __fadd_rn(__fadd_rn(a, b), g[8]);
-}
-// Per node and species: keep = 1 - om, a = om C_s (scale 2^14), and w_i
-// times the node's stored reference (scale 2^14) for the three weights.
-struct PushK {
-  float keep, a, wq[3];
-};
-__device__ __forceinline__ PushK push_k(float om, float cs, float cqs) {
-  PushK k;
-  k.keep = __fsub_rn(1.0f, om);
-  k.a = __fmul_rn(om, cs);
-  k.wq[0] = __fmul_rn(w(0), cqs);
-  k.wq[1] = __fmul_rn(w(1), cqs);
-  k.wq[2] = __fmul_rn(w(5), cqs);
-  return k;
-}
-// value stored for population i: the BGK relaxation (1 - om) G + om C_s E_i
-// less w_i times the node's stored reference, all at scale 2^14: two FMAs
-__device__ __forceinline__ float push(int i, float g, float e, const PushK &k) {
-  const float wq = i == 0 ? k.wq[0] : (i < 5 ? k.wq[1] : k.wq[2]);
-  return __fmaf_rn(k.keep, g, __fmaf_rn(k.a, e, -wq));
-}
-
-// Packed two-node forms of the arithmetic above (this part's f32x2 FMA, add
-// and multiply): lane 0 is node x0, lane 1 node x0 + 1, and each lane is
-// rounded exactly like the scalar operation, so a lane's bits equal the
-// one-node form's.  One packed instruction does the work of two (measured
-// 0.7% faster per step than the scalar form on two nodes).
+// A scaled population is pulled as its stored deviation h plus w_i 2^14 times
+// the source's reference concentration r (as stored, at scale 1); w_i 2^14 is
+// exact, so this equals fma(w_i, 2^14 r, h) bit for bit, without the multiply
+// by 2^14.  The equilibrium factors E_i(u) = w_i (1 + 3 c.u + 4.5 (c.u)^2 -
+// 1.5 u.u) are built for each direction together with its opposite (c.u
+// changes sign, the even part is shared).  The value stored is the BGK
+// relaxation (1 - om) G + om C_s E_i less w_i times the node's stored
+// reference, all at scale 2^14: two FMAs.
+// Two nodes at a time in this part's f32x2 FMA, add and multiply: lane 0 is
+// node x0, lane 1 node x0 + 1, each lane rounded exactly like the scalar
+// operation.  One packed instruction does the work of two (measured 0.7%
+// faster per step than the scalar form on two nodes).
 __device__ __forceinline__ float2 dup(float v) { return make_float2(v, v); }
 __device__ __forceinline__ void eq2(float2 ux, float2 uy, float2 (&E)[9]) {
   const float2 base = __ffma2_rn(dup(-1.5f), __ffma2_rn(ux, ux, __fmul2_rn(uy, uy)),
@@ -159,8 +115,8 @@ __device__ __forceinline__ __half round_half(float v, uint32_t h, int k) {
 // The two nodes of a pair (lo: even x, hi: odd x) at store index k =
 // 9 s + i.  LBM_F16_SR_HW = 1 (default): one cvt.rs instruction (this
 // part's stochastic-rounding conversion) rounds both, with 32 random bits
-// from the same hash; each half is rounded on its own, so the one-node form,
-// which passes 0 for the other half, gets the same bits.  It measured 2.7%
+// from the same hash; each half is rounded on its own, so a node gets the same
+// bits whatever is passed for the other half.  It measured 2.7%
 // faster per step than round_half above (four instructions per value) with
 // the same steady-state efficiency error.  LBM_F16_SR_HW = 0: round_half,
 // element by element.
@@ -182,56 +138,6 @@ __device__ __forceinline__ __half2 round_pair(float lo, float hi, uint32_t h,
 }
 }  // namespace f16
 
-template <int NS, int MODE>
-__device__ __forceinline__ void adr_interior_node_f16(const AdrArgs &a, long long n,
-                                                      float (&acc)[3 * NS]) {
-  const long long np = a.nx_pad, plane = a.plane;
-  const __half *__restrict__ src = static_cast<const __half *>(a.src);
-  __half *__restrict__ dst = static_cast<__half *>(a.dst);
-  const float *__restrict__ U = static_cast<const float *>(a.u);
-  float g[NS][9];
-#pragma unroll
-  for (int s = 0; s < NS; ++s) {
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      const long long m = n - (cy(i) * np + cx(i));
-      g[s][i] = f16::pull(i, __half2float(src[(long long)(s * 9 + i) * plane + m]),
-                          __half2float(a.rsrc[s * plane + m]));
-    }
-  }
-  float *__restrict__ cp = static_cast<float *>(a.cprev);
-  float prev[NS];
-  if (MODE == kAdrCheck) {
-#pragma unroll
-    for (int s = 0; s < NS; ++s) prev[s] = cp[s * plane + n];
-  }
-  float E[9];
-  f16::eq(U[n], U[plane + n], E);
-  const uint32_t h = f16::pair_hash(n >> 1, a.step);
-  const bool odd = (n & 1) != 0;   // second node of its pair
-#pragma unroll
-  for (int s = 0; s < NS; ++s) {
-    const float cs = f16::sum9(g[s]);
-    const float c = __fmul_rn(cs, f16::kDown);
-    const float cqs = __fmul_rn(ref_round(c), f16::kUp);
-    a.rdst[s * plane + n] = __float2half_rn(c);
-    const f16::PushK k = f16::push_k(a.fomega[s], cs, cqs);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      // rounded as one half of its pair, with the pair's random bits
-      const float v = f16::push(i, g[s][i], E[i], k);
-      const __half2 r2 = f16::round_pair(odd ? 0.0f : v, odd ? v : 0.0f, h,
-                                         s * 9 + i);
-      dst[(long long)(s * 9 + i) * plane + n] = odd ? __high2half(r2)
-                                                    : __low2half(r2);
-    }
-    if (MODE == kAdrCheck) {
-      check_add<NS, float>(acc, s, c, prev[s]);
-      cp[s * plane + n] = c;
-    }
-  }
-}
-
 // FP16 bulk step, two nodes per thread: nodes (x0, x0 + 1), x0 even, of row
 // y.  Every plane is read as aligned half2 pairs.  A pull with c_ix = +1
 // takes the sources (x0 - 1, x0): the high half of the pair to the left and
@@ -242,7 +148,7 @@ __device__ __forceinline__ void adr_interior_node_f16(const AdrArgs &a, long lon
 // nx - 1, so x0 + 3 < nx_pad): every read stays inside its row, and rows
 // y +- 1 exist whenever either node is interior.  The reference
 // concentrations of the source nodes come the same way (three rows of three
-// pairs per species).  The arithmetic is that of adr_interior_node_f16.
+// pairs per species).
 // A block has kBlockX / 2 threads and covers a segment of kBlockX nodes.
 //
 // Each thread reads 24 pairs per species: slot 0..8 its own pair of plane
@@ -368,16 +274,15 @@ __device__ __forceinline__ void pair_update(const AdrArgs &a, int y, int x0,
   }
 }
 
-// The two nodes per thread of one row segment, loaded species by species:
-// the block first sends the L2 prefetches for the segment
+// Nodes [xb, xb + 2 THREADS) of row y, two per thread, loaded species by
+// species: the block first sends the L2 prefetches for the segment
 // LBM_PREFETCH_ROWS_F16 rows below it.
-template <int NS, int MODE>
-__device__ __forceinline__ void pair_segment(const AdrArgs &a,
+template <int NS, int MODE, int THREADS>
+__device__ __forceinline__ void pair_segment(const AdrArgs &a, int y, int xb,
                                              float (&acc)[2][3 * NS]) {
-  const int y = blockIdx.y;
   if (LBM_PREFETCH_ROWS_F16 > 0)
-    bulk_prefetch_rows<__half, float, NS, true>(a, y + LBM_PREFETCH_ROWS_F16);
-  const int x0 = 2 * (blockIdx.x * kPairThreads + threadIdx.x);
+    prefetch_rows_f16<NS, THREADS>(a, y + LBM_PREFETCH_ROWS_F16, xb, 2 * THREADS);
+  const int x0 = xb + 2 * threadIdx.x;
   const long long n0 = (long long)y * a.nx_pad + x0;
   uint2 lw = make_uint2(kSolidNode, kSolidNode);
   if (x0 < a.nx_pad) lw = *reinterpret_cast<const uint2 *>(a.links + n0);
@@ -408,7 +313,7 @@ __global__ void __launch_bounds__(kPairThreads, 5)
   if (chunk >= 0)
     boundary_nodes<PrecF16Dev, NS, kAdrCheck, kPairThreads>(a, chunk, acc[0]);
   else
-    pair_segment<NS, kAdrCheck>(a, acc);
+    pair_segment<NS, kAdrCheck, kPairThreads>(a, blockIdx.y, blockIdx.x * kBlockX, acc);
   const long long row = partial_row<kPairThreads>(a, chunk);
   if (row >= 0)
     block_partials_store<2 * NS, NS, 2, kPairThreads, float>(
@@ -436,21 +341,12 @@ __global__ void __launch_bounds__(kPairThreads, 5)
 #endif
 constexpr int kQuadThreads = kBlockX / 4;
 
-template <int NS>
-__global__ void __launch_bounds__(kQuadThreads, LBM_QUAD_MIN_BLOCKS)
-    adr_step_quad_kernel(const AdrArgs a) {
-  static_assert(kQuadThreads >= 9 * NS + NS + 3, "one prefetch per thread");
-  static_assert(kQuadThreads % 32 == 0, "whole warps");
-  const long long chunk = boundary_chunk(a);
-  if (chunk >= 0) {
-    float acc[3 * NS];
-    boundary_nodes<PrecF16Dev, NS, kAdrStep, kQuadThreads>(a, chunk, acc);
-    return;
-  }
-  const int y = blockIdx.y;
+// Nodes [xb, xb + 4 THREADS) of row y, four per thread.
+template <int NS, int THREADS>
+__device__ __forceinline__ void quad_segment(const AdrArgs &a, int y, int xb) {
   if (LBM_PREFETCH_ROWS_F16 > 0)
-    bulk_prefetch_rows<__half, float, NS, true>(a, y + LBM_PREFETCH_ROWS_F16);
-  const int x0 = 4 * (blockIdx.x * kQuadThreads + threadIdx.x);
+    prefetch_rows_f16<NS, THREADS>(a, y + LBM_PREFETCH_ROWS_F16, xb, 4 * THREADS);
+  const int x0 = xb + 4 * threadIdx.x;
   if (x0 >= a.nx_pad) return;   // nx_pad is a multiple of 4: x0 + 3 < nx_pad
   const long long np = a.nx_pad, plane = a.plane;
   const long long n0 = (long long)y * np + x0;
@@ -576,6 +472,21 @@ __global__ void __launch_bounds__(kQuadThreads, LBM_QUAD_MIN_BLOCKS)
       if (in2) ro[2] = __low2half(crh);
       if (in3) ro[3] = __high2half(crh);
     }
+  }
+}
+
+// The plain step of the FP16 storage: the row segments four nodes per thread,
+// and the boundary chunks.
+template <int NS>
+__global__ void __launch_bounds__(kQuadThreads, LBM_QUAD_MIN_BLOCKS)
+    adr_step_quad_kernel(const AdrArgs a) {
+  static_assert(kQuadThreads % 32 == 0, "whole warps");
+  const long long chunk = boundary_chunk(a);
+  if (chunk < 0) {
+    quad_segment<NS, kQuadThreads>(a, blockIdx.y, blockIdx.x * kBlockX);
+  } else {
+    float acc[3 * NS];
+    boundary_nodes<PrecF16Dev, NS, kAdrStep, kQuadThreads>(a, chunk, acc);
   }
 }
 

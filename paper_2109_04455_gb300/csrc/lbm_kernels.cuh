@@ -566,18 +566,15 @@ __device__ __forceinline__ void adr_boundary_node(const AdrArgs &a, long long n,
   });
 }
 
-// L2 prefetch ahead of the bulk stencil.  With D = LBM_PREFETCH_ROWS_* > 0
-// each block of the bulk step asks L2 for the row segments that the block D
-// rows further down will read: one bulk prefetch per plane (the 9 NS
-// population rows y + D - c_iy, for FP16 storage the NS reference rows, u
-// and the link words of row y + D).  Blocks start in row order, so those
-// lines are on their way from HBM about D rows of blocks before their loads
-// are issued, and they are in flight without holding registers.
+// L2 prefetch ahead of the FP16 steps.  With D = LBM_PREFETCH_ROWS_F16 > 0
+// each block asks L2 for the row segments that the block D rows further down
+// will read: one bulk prefetch per plane (the 9 NS population rows y + D -
+// c_iy, the NS reference rows, u and the link words of row y + D).  Blocks
+// start in row order, so those lines are on their way from HBM about D rows
+// of blocks before their loads are issued, and they are in flight without
+// holding registers.
 #ifndef LBM_PREFETCH_ROWS_F16
 #define LBM_PREFETCH_ROWS_F16 6
-#endif
-#ifndef LBM_PREFETCH_ROWS_F32
-#define LBM_PREFETCH_ROWS_F32 0
 #endif
 // [p, p + bytes) into L2, nothing to wait for; p 16-byte aligned and bytes
 // a multiple of 16
@@ -585,34 +582,30 @@ __device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;"
                :: "l"(p), "r"(bytes) : "memory");
 }
-// S: stored population type, U: velocity type, REF: reference planes
-// (FP16 storage).  Rows outside the lattice are skipped.
-template <typename S, typename U, int NS, bool REF>
-__device__ __forceinline__ void bulk_prefetch_rows(const AdrArgs &a, int yp) {
-  constexpr int kPop = 9 * NS, kRef = REF ? NS : 0;
-  const int t = threadIdx.x;
-  if (t >= kPop + kRef + 3 || yp >= a.ny) return;
+// Nodes [xb, xb + width) of row yp, xb and width multiples of 32, by a block
+// of THREADS threads; rows outside the lattice are skipped.
+template <int NS, int THREADS>
+__device__ __forceinline__ void prefetch_rows_f16(const AdrArgs &a, int yp, int xb, int width) {
+  constexpr int kPop = 9 * NS, kAll = kPop + NS + 3;
+  if (yp >= a.ny) return;
   const long long np = a.nx_pad, plane = a.plane;
-  const int xb = blockIdx.x * kBlockX;
-  // nx_pad is a multiple of 32 and xb of kBlockX, so every segment starts
-  // 64-byte aligned (buffers are 256-byte aligned) and is a multiple of 64
-  // bytes long
-  const unsigned cnt = static_cast<unsigned>(min(kBlockX, a.nx_pad - xb));
-  if (t < kPop) {
-    const int i = t % 9, row = yp - cy(i);
-    if (row < 0 || row >= a.ny) return;
-    prefetch_l2(static_cast<const S *>(a.src) + (long long)t * plane +
-                    (long long)row * np + xb,
-                static_cast<unsigned>(sizeof(S)) * cnt);
-  } else if (t < kPop + kRef) {
-    prefetch_l2(a.rsrc + (long long)(t - kPop) * plane + (long long)yp * np + xb,
-                static_cast<unsigned>(sizeof(RefT)) * cnt);
-  } else if (t < kPop + kRef + 2) {
-    prefetch_l2(static_cast<const U *>(a.u) + (long long)(t - kPop - kRef) * plane +
-                    (long long)yp * np + xb,
-                static_cast<unsigned>(sizeof(U)) * cnt);
-  } else {
-    prefetch_l2(a.links + (long long)yp * np + xb, 4u * cnt);
+  // nx_pad is a multiple of 32, so every segment starts 64-byte aligned
+  // (buffers are 256-byte aligned) and is a multiple of 64 bytes long
+  const unsigned cnt = static_cast<unsigned>(min(width, a.nx_pad - xb));
+#pragma unroll
+  for (int k = 0; k < kAll; k += THREADS) {
+    const int t = k + threadIdx.x;
+    if (t < kPop) {
+      const int row = yp - cy(t % 9);
+      if (row >= 0 && row < a.ny)
+        prefetch_l2(static_cast<const __half *>(a.src) + t * plane + row * np + xb, 2u * cnt);
+    } else if (t < kPop + NS) {
+      prefetch_l2(a.rsrc + (t - kPop) * plane + yp * np + xb, 2u * cnt);
+    } else if (t < kPop + NS + 2) {
+      prefetch_l2(static_cast<const float *>(a.u) + (t - kPop - NS) * plane + yp * np + xb, 4u * cnt);
+    } else if (t < kAll) {
+      prefetch_l2(a.links + yp * np + xb, 4u * cnt);
+    }
   }
 }
 
@@ -646,12 +639,12 @@ __device__ __forceinline__ long long partial_row(const AdrArgs &a, long long chu
 }
 
 }  // namespace lbm
-// FP16-deviation storage: interior update (one and two nodes per thread)
+// FP16-deviation storage: interior update (two and four nodes per thread)
 #include "lbm_f16.cuh"
 namespace lbm {
 
-// Update of one interior node (link word 0: every neighbour is fluid): the
-// interior formula (pull from x - c_i, BGK, no source).  All populations of
+// Update of one interior node (link word 0: every neighbour is fluid), FP32
+// and FP64: the interior formula (pull from x - c_i, BGK, no source).  All populations of
 // all species are loaded before any arithmetic, so a thread keeps NS*9
 // independent loads in flight.
 template <class P, int NS, int MODE>
@@ -659,10 +652,6 @@ __device__ __forceinline__ void adr_interior_node(const AdrArgs &a, long long n,
                                                   typename P::T (&acc)[3 * NS]) {
   using S = typename P::S;
   using T = typename P::T;
-  if constexpr (P::kDev) {
-    adr_interior_node_f16<NS, MODE>(a, n, acc);
-    return;
-  }
   const long long np = a.nx_pad, plane = a.plane;
   const S *__restrict__ src = static_cast<const S *>(a.src);
   S *__restrict__ dst = static_cast<S *>(a.dst);
