@@ -3,14 +3,15 @@
 
 namespace lbm {
 template cudaError_t launch_adr<PrecF64>(int, int, const AdrArgs &,
-                                            cudaStream_t);
+                                            cudaStream_t, bool);
 template cudaError_t launch_adr_flux<PrecF64>(int, const void *, const RefT *,
                                                  const uint32_t *, long long,
                                                  int, int, int, double *,
                                                  cudaStream_t);
-template cudaError_t launch_flow<PrecF64>(int, const FlowArgs &, cudaStream_t);
+template cudaError_t launch_flow<PrecF64>(int, const FlowArgs &, cudaStream_t,
+                                          bool);
 template cudaError_t launch_adjoint<PrecF64>(int, int, const AdjArgs &,
-                                                cudaStream_t);
+                                                cudaStream_t, bool);
 template cudaError_t launch_adjoint_grad<PrecF64>(
     int, const AdjArgs &, const BoundaryNode *, long long, const void *, double *,
     double *, const int32_t *, double *, double, double, cudaStream_t);

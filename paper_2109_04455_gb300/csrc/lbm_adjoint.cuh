@@ -131,6 +131,7 @@ __global__ void __launch_bounds__(kBlockX) adj_kernel(const AdjArgs a) {
   const long long plane = a.plane;
   const uint32_t lw = (x < a.nx_pad) ? a.links[n] : kSolidNode;
   T acc[2] = {T(0), T(0)};
+  wait_for_previous();
   if (lw == 0u) {
     const long long np = a.nx_pad;
     const T *nu = static_cast<const T *>(a.src);

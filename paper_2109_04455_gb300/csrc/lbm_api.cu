@@ -158,9 +158,9 @@ extern "C" size_t lbm_flow_ws_bytes(const lbm_geometry *g, int32_t precision) {
 }
 
 static cudaError_t flow_launch(int prec, int mode, const FlowArgs &a,
-                               cudaStream_t st) {
-  return prec == LBM_F64 ? launch_flow<PrecF64>(mode, a, st)
-                         : launch_flow<PrecF32>(mode, a, st);
+                               cudaStream_t st, bool chained) {
+  return prec == LBM_F64 ? launch_flow<PrecF64>(mode, a, st, chained)
+                         : launch_flow<PrecF32>(mode, a, st, chained);
 }
 
 extern "C" lbm_status lbm_flow_solve(const lbm_geometry *g,
@@ -236,28 +236,28 @@ extern "C" lbm_status lbm_flow_solve(const lbm_geometry *g,
   if (e != cudaSuccess) return cuda_fail("lbm_flow_solve", e);
   a.src = nullptr;
   a.dst = buf[0];
-  e = flow_launch(prec, kFlowInit, a, st);
+  e = flow_launch(prec, kFlowInit, a, st, false);
   if (e != cudaSuccess) return cuda_fail("lbm_flow_solve(init)", e);
   int cur = 0;
   int64_t steps = 0;
   double residual = INFINITY;
   bool converged = false;
 
-  auto step = [&](int mode) -> cudaError_t {
+  auto step = [&](int mode, bool chained) -> cudaError_t {
     a.src = buf[cur];
     a.dst = buf[cur ^ 1];
     cur ^= 1;
     ++steps;
-    return flow_launch(prec, mode, a, st);
+    return flow_launch(prec, mode, a, st, chained);
   };
   // n steps, the last two writing u and the residual sums
   auto chunk = [&](int64_t n) -> lbm_status {
     for (int64_t k = 0; k < n - 2; ++k) {
-      cudaError_t e2 = step(kFlowStep);
+      cudaError_t e2 = step(kFlowStep, k > 0);
       if (e2 != cudaSuccess) return cuda_fail("lbm_flow_solve(step)", e2);
     }
-    cudaError_t e2 = step(kFlowU);
-    if (e2 == cudaSuccess) e2 = step(kFlowCheck);
+    cudaError_t e2 = step(kFlowU, n > 2);
+    if (e2 == cudaSuccess) e2 = step(kFlowCheck, true);
     if (e2 == cudaSuccess)
       e2 = launch_reduce(2, 0, partials, flow_blocks(g), scratch, result, st);
     double h[2] = {0, 0};
@@ -362,11 +362,11 @@ extern "C" size_t lbm_adr_ws_bytes(const lbm_geometry *g,
 }
 
 static cudaError_t adr_launch(int prec, int ns, int mode, const AdrArgs &a,
-                              cudaStream_t st) {
+                              cudaStream_t st, bool chained = false) {
   switch (prec) {
-    case LBM_F64: return launch_adr<PrecF64>(ns, mode, a, st);
-    case LBM_F32: return launch_adr<PrecF32>(ns, mode, a, st);
-    default: return launch_adr<PrecF16Dev>(ns, mode, a, st);
+    case LBM_F64: return launch_adr<PrecF64>(ns, mode, a, st, chained);
+    case LBM_F32: return launch_adr<PrecF32>(ns, mode, a, st, chained);
+    default: return launch_adr<PrecF16Dev>(ns, mode, a, st, chained);
   }
 }
 
@@ -525,8 +525,9 @@ static AdrArgs adr_next(lbm_adr_solver *s, int steps) {
   return a;
 }
 
-static cudaError_t adr_step(lbm_adr_solver *s, int mode, cudaStream_t st) {
-  return adr_launch(s->p.precision, s->p.nspecies, mode, adr_next(s, 1), st);
+// chained: after another step of this run (see launch_chained)
+static cudaError_t adr_step(lbm_adr_solver *s, int mode, cudaStream_t st, bool chained) {
+  return adr_launch(s->p.precision, s->p.nspecies, mode, adr_next(s, 1), st, chained);
 }
 
 // n plain steps
@@ -538,7 +539,7 @@ static cudaError_t adr_plain_steps(lbm_adr_solver *s, int64_t n, cudaStream_t st
       e = launch_adr_two_step(s->p.nspecies, adr_next(s, 2), st);
       k += 2;
     } else {
-      e = adr_step(s, kAdrStep, st);
+      e = adr_step(s, kAdrStep, st, k > 0);
       k += 1;
     }
   }
@@ -559,8 +560,8 @@ extern "C" lbm_status lbm_adr_run(lbm_adr_solver *s, int64_t nsteps,
   cudaError_t e = adr_plain_steps(s, plain, st);
   if (e != cudaSuccess) return cuda_fail("lbm_adr_run(step)", e);
   if (!info) return LBM_OK;
-  e = adr_step(s, kAdrCheck, st);
-  if (e == cudaSuccess) e = adr_step(s, kAdrCheck, st);
+  e = adr_step(s, kAdrCheck, st, plain > 0);
+  if (e == cudaSuccess) e = adr_step(s, kAdrCheck, st, true);
   if (e == cudaSuccess)
     e = launch_reduce(2 * ns, ns, s->partials, s->nb, s->scratch, s->result, st);
   if (e == cudaSuccess) e = adr_flux_launch(s, st);
@@ -816,9 +817,9 @@ extern "C" size_t lbm_adr_adjoint_ws_bytes(const lbm_geometry *g,
 }
 
 static cudaError_t adj_launch(int prec, int ns, int mode, const AdjArgs &a,
-                              cudaStream_t st) {
-  return prec == LBM_F64 ? launch_adjoint<PrecF64>(ns, mode, a, st)
-                         : launch_adjoint<PrecF32>(ns, mode, a, st);
+                              cudaStream_t st, bool chained) {
+  return prec == LBM_F64 ? launch_adjoint<PrecF64>(ns, mode, a, st, chained)
+                         : launch_adjoint<PrecF32>(ns, mode, a, st, chained);
 }
 
 // d eps / d N_s of Eq. (A-B)
@@ -932,7 +933,7 @@ extern "C" lbm_status lbm_adr_adjoint(lbm_adr_solver *s, int64_t max_steps,
       a.src = buf[cur];
       a.dst = buf[cur ^ 1];
       const int mode = (k == n - 1) ? kAdjCheck : kAdjStep;
-      cudaError_t e2 = adj_launch(prec, ns, mode, a, st);
+      cudaError_t e2 = adj_launch(prec, ns, mode, a, st, k > 0);
       if (e2 != cudaSuccess) return cuda_fail("lbm_adr_adjoint(step)", e2);
       cur ^= 1;
       ++steps;

@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(StepThreads<P, MODE, TILE>::value,
         const int x = x0 + threadIdx.x;
         const long long n = (long long)y * sa.nx_pad + x;
         const uint32_t lw = (x < sa.nx_pad) ? sa.links[n] : kSolidNode;
-        if (lw == 0u) adr_interior_node<P, NS, MODE>(sa, n, acc[0]);
+        if (lw == 0u) adr_interior_node<P, NS, MODE, false>(sa, n, acc[0]);
       }
     } else {
       const long long t =

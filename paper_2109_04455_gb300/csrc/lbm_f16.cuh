@@ -288,6 +288,7 @@ __device__ __forceinline__ void pair_segment(const AdrArgs &a, int y, int xb,
   if (x0 < a.nx_pad) lw = *reinterpret_cast<const uint2 *>(a.links + n0);
   const bool in0 = lw.x == 0u, in1 = lw.y == 0u;
   if (!in0 && !in1) return;
+  wait_for_previous();
   const __half2 z2 = __float2half2_rn(0.0f);
   const float *__restrict__ U = static_cast<const float *>(a.u);
   const float2 ux = *reinterpret_cast<const float2 *>(U + n0);
@@ -314,6 +315,7 @@ __global__ void __launch_bounds__(kPairThreads, 5)
     boundary_nodes<PrecF16Dev, NS, kAdrCheck, kPairThreads>(a, chunk, acc[0]);
   else
     pair_segment<NS, kAdrCheck, kPairThreads>(a, blockIdx.y, blockIdx.x * kBlockX, acc);
+  wait_for_previous();   // the partial sums are one buffer
   const long long row = partial_row<kPairThreads>(a, chunk);
   if (row >= 0)
     block_partials_store<2 * NS, NS, 2, kPairThreads, float>(
@@ -366,6 +368,7 @@ __device__ __forceinline__ void quad_segment(const AdrArgs &a, int y, int xb) {
   const uint32_t hl = f16::pair_hash(n0 >> 1, a.step);
   const uint32_t hh = f16::pair_hash((n0 >> 1) + 1, a.step);
   const __half hz = __float2half_rn(0.0f);
+  wait_for_previous();
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
     // the species' loads, issued before its arithmetic: nine own quads,

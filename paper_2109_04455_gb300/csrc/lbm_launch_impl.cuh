@@ -8,44 +8,42 @@
 namespace lbm {
 
 template <class P, int NS, int MODE>
-static void launch_step(AdrArgs a, cudaStream_t st) {
+static cudaError_t launch_step(AdrArgs a, cudaStream_t st, bool chained) {
   if constexpr (P::kDev) {
     constexpr int kThreads = MODE == kAdrCheck ? kPairThreads : kQuadThreads;
     const AdrGrid g = adr_grid(a.nx_pad, a.ny, a.nbnd, kBlockX, kThreads);
     a.nxb = g.nxb;
     if constexpr (MODE == kAdrCheck)
-      adr_check_pair_kernel<NS><<<g.grid, kThreads, 0, st>>>(a);
+      return launch_chained(chained, adr_check_pair_kernel<NS>, g.grid, kThreads, st, a);
     else
-      adr_step_quad_kernel<NS><<<g.grid, kThreads, 0, st>>>(a);
+      return launch_chained(chained, adr_step_quad_kernel<NS>, g.grid, kThreads, st, a);
   } else {
     const int bx = adr_block_x(sizeof(typename P::S) == 8 ? LBM_F64 : LBM_F32,
                                a.nx_pad, a.ny);
     const AdrGrid g = adr_grid(a.nx_pad, a.ny, a.nbnd, bx, bx);
     a.nxb = g.nxb;
-    if (bx == 64)
-      adr_step_kernel<P, NS, MODE, 64><<<g.grid, 64, 0, st>>>(a);
-    else
-      adr_step_kernel<P, NS, MODE, 256><<<g.grid, 256, 0, st>>>(a);
+    return launch_chained(chained, bx == 64 ? adr_step_kernel<P, NS, MODE, 64>
+                                            : adr_step_kernel<P, NS, MODE, 256>,
+                          g.grid, bx, st, a);
   }
 }
 
 template <class P, int NS>
-static cudaError_t launch_adr_ns(int mode, const AdrArgs &a, cudaStream_t st) {
-  if (mode == kAdrInit)
-    adr_init_kernel<P, NS><<<adr_node_grid(a.nx_pad, a.ny), kBlockX, 0, st>>>(a);
-  else if (mode == kAdrStep)
-    launch_step<P, NS, kAdrStep>(a, st);
-  else
-    launch_step<P, NS, kAdrCheck>(a, st);
+static cudaError_t launch_adr_ns(int mode, const AdrArgs &a, cudaStream_t st,
+                                 bool chained) {
+  if (mode == kAdrStep) return launch_step<P, NS, kAdrStep>(a, st, chained);
+  if (mode == kAdrCheck) return launch_step<P, NS, kAdrCheck>(a, st, chained);
+  adr_init_kernel<P, NS><<<adr_node_grid(a.nx_pad, a.ny), kBlockX, 0, st>>>(a);
   return cudaGetLastError();
 }
 
 template <class P>
-cudaError_t launch_adr(int ns, int mode, const AdrArgs &a, cudaStream_t st) {
+cudaError_t launch_adr(int ns, int mode, const AdrArgs &a, cudaStream_t st,
+                       bool chained) {
   switch (ns) {
-    case 1: return launch_adr_ns<P, 1>(mode, a, st);
-    case 2: return launch_adr_ns<P, 2>(mode, a, st);
-    case 3: return launch_adr_ns<P, 3>(mode, a, st);
+    case 1: return launch_adr_ns<P, 1>(mode, a, st, chained);
+    case 2: return launch_adr_ns<P, 2>(mode, a, st, chained);
+    case 3: return launch_adr_ns<P, 3>(mode, a, st, chained);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -67,49 +65,41 @@ cudaError_t launch_adr_flux(int ns, const void *g, const RefT *ref,
 }
 
 template <class P, int BX>
-static cudaError_t launch_flow_bx(int mode, const FlowArgs &a, cudaStream_t st) {
-  const dim3 grid = flow_grid(a.nx_pad, a.ny);
-  switch (mode) {
-    case kFlowStep: flow_kernel<P, kFlowStep, BX><<<grid, BX, 0, st>>>(a); break;
-    case kFlowU: flow_kernel<P, kFlowU, BX><<<grid, BX, 0, st>>>(a); break;
-    case kFlowCheck: flow_kernel<P, kFlowCheck, BX><<<grid, BX, 0, st>>>(a); break;
-    case kFlowInit: flow_kernel<P, kFlowInit, BX><<<grid, BX, 0, st>>>(a); break;
+static cudaError_t launch_flow_bx(int mode, const FlowArgs &a, cudaStream_t st,
+                                  bool chained) {
+  const auto kernel = mode == kFlowStep ? flow_kernel<P, kFlowStep, BX>
+                      : mode == kFlowU  ? flow_kernel<P, kFlowU, BX>
+                      : mode == kFlowCheck ? flow_kernel<P, kFlowCheck, BX>
+                                           : flow_kernel<P, kFlowInit, BX>;
+  return launch_chained(chained, kernel, flow_grid(a.nx_pad, a.ny), BX, st, a);
+}
+
+template <class P>
+cudaError_t launch_flow(int mode, const FlowArgs &a, cudaStream_t st, bool chained) {
+  return flow_block_x(a.nx_pad, a.ny) == 64 ? launch_flow_bx<P, 64>(mode, a, st, chained)
+                                            : launch_flow_bx<P, 256>(mode, a, st, chained);
+}
+
+template <class P, int NS>
+static cudaError_t launch_adjoint_ns(int mode, const AdjArgs &a, cudaStream_t st,
+                                     bool chained) {
+  using T = typename P::T;
+  const auto kernel = mode == kAdjCheck ? (a.periodic ? adj_kernel<T, NS, kAdjCheck, true>
+                                                      : adj_kernel<T, NS, kAdjCheck, false>)
+                                        : (a.periodic ? adj_kernel<T, NS, kAdjStep, true>
+                                                      : adj_kernel<T, NS, kAdjStep, false>);
+  return launch_chained(chained, kernel, adr_node_grid(a.nx_pad, a.ny), kBlockX, st, a);
+}
+
+template <class P>
+cudaError_t launch_adjoint(int ns, int mode, const AdjArgs &a, cudaStream_t st,
+                           bool chained) {
+  switch (ns) {
+    case 1: return launch_adjoint_ns<P, 1>(mode, a, st, chained);
+    case 2: return launch_adjoint_ns<P, 2>(mode, a, st, chained);
+    case 3: return launch_adjoint_ns<P, 3>(mode, a, st, chained);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
-}
-
-template <class P>
-cudaError_t launch_flow(int mode, const FlowArgs &a, cudaStream_t st) {
-  return flow_block_x(a.nx_pad, a.ny) == 64 ? launch_flow_bx<P, 64>(mode, a, st)
-                                            : launch_flow_bx<P, 256>(mode, a, st);
-}
-
-template <class P>
-cudaError_t launch_adjoint(int ns, int mode, const AdjArgs &a, cudaStream_t st) {
-  using T = typename P::T;
-  const dim3 block(kBlockX);
-  const dim3 grid = adr_node_grid(a.nx_pad, a.ny);
-#define LBM_ADJ_CASE(NS)                                                  \
-  if (ns == NS) {                                                         \
-    if (mode == kAdjCheck) {                                              \
-      if (a.periodic)                                                     \
-        adj_kernel<T, NS, kAdjCheck, true><<<grid, block, 0, st>>>(a);    \
-      else                                                                \
-        adj_kernel<T, NS, kAdjCheck, false><<<grid, block, 0, st>>>(a);   \
-    } else {                                                              \
-      if (a.periodic)                                                     \
-        adj_kernel<T, NS, kAdjStep, true><<<grid, block, 0, st>>>(a);     \
-      else                                                                \
-        adj_kernel<T, NS, kAdjStep, false><<<grid, block, 0, st>>>(a);    \
-    }                                                                     \
-    return cudaGetLastError();                                            \
-  }
-  LBM_ADJ_CASE(1)
-  LBM_ADJ_CASE(2)
-  LBM_ADJ_CASE(3)
-#undef LBM_ADJ_CASE
-  return cudaErrorInvalidValue;
 }
 
 template <class P>

@@ -62,31 +62,6 @@ __device__ __forceinline__ void edge_mask_rules(uint32_t mask, float v, float (&
     if (mask >> i & 1u) g[i] = fma_rn(2.0f * Lattice<float>::w(i), v, -g[i]);
 }
 
-// whether node (x, y), link word lw, has catalytic links, and their rates,
-// all loaded at once
-__device__ __forceinline__ bool link_rates(const AdrArgs &a, uint32_t lw, int x, int y,
-                                           float (&ka)[9], float (&kb)[9]) {
-  bool cat = false;
-#pragma unroll
-  for (int j = 1; j < 9; ++j) cat = cat || nib(lw, j) == kCat;
-  if (cat) {
-    double da[9], db[9];
-#pragma unroll
-    for (int j = 1; j < 9; ++j) {
-      const bool on = nib(lw, j) == kCat;
-      const long long m = on ? neighbour(x, y, j, a.nx, a.ny, a.nx_pad) : 0;
-      da[j] = on ? a.kab[m] : 0.0;
-      db[j] = on ? a.kbc[m] : 0.0;
-    }
-#pragma unroll
-    for (int j = 1; j < 9; ++j) {
-      ka[j] = float(da[j]);
-      kb[j] = float(db[j]);
-    }
-  }
-  return cat;
-}
-
 template <int NS>
 __global__ void __launch_bounds__(TwoStep<NS>::kBX, TwoStep<NS>::kBlocks)
     adr_two_step_kernel(const AdrArgs a, int rows) {
