@@ -225,11 +225,7 @@ extern "C" lbm_status lbm_flow_solve(const lbm_geometry *g,
   a.k3 = 3.0 * a.k1;
   a.k45 = 4.5 * a.k1;
   a.u0 = p->u0;
-  a.fkeep = static_cast<float>(a.keep);
-  a.fkh = static_cast<float>(a.kh);
-  a.fk1 = static_cast<float>(a.k1);
-  a.fk3 = static_cast<float>(a.k3);
-  a.fk45 = static_cast<float>(a.k45);
+  a.fomega = static_cast<float>(om);
   a.fu0 = static_cast<float>(a.u0);
 
   cudaError_t e = cudaMemsetAsync(b, 0, 2 * bufb, st);

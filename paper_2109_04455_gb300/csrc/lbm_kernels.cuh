@@ -883,7 +883,7 @@ struct FlowArgs {
   double keep, kh;        // 1 - 1/tau, and half of it
   double k1, k3, k45;     // k1 = 1/(9 tau), 3 k1, 4.5 k1
   double u0;              // inflow centreline velocity
-  float fkeep, fkh, fk1, fk3, fk45, fu0;   // the same in float
+  float fomega, fu0;      // 1/tau and u0 in float
 };
 
 enum FlowMode { kFlowStep = 0, kFlowU = 1, kFlowCheck = 2, kFlowInit = 3 };
@@ -893,7 +893,6 @@ enum FlowMode { kFlowStep = 0, kFlowU = 1, kFlowCheck = 2, kFlowInit = 3 };
 // division's, to within an ulp of it.  The conversions to float and back are
 // shifts of the bit patterns (they would be FP64 operations too).  Values
 // outside 2^-60 .. 2^60 (a lattice that diverges) are divided.
-__device__ __forceinline__ float reciprocal(float v) { return 1.0f / v; }
 __device__ __forceinline__ double reciprocal(double v) {
   const unsigned hi = __double2hiint(v), lo = __double2loint(v);
   const unsigned sign = hi & 0x80000000u, mag = hi & 0x7FFFFFFFu;
@@ -984,9 +983,8 @@ __global__ void __launch_bounds__(BX) flow_kernel(const FlowArgs a) {
           jx += T(cx(j)) * own[j];
           jy += T(cy(j)) * own[j];
         }
-        const T q = reciprocal(r);
-        uwx = jx * q;
-        uwy = jy * q;
+        uwx = jx / r;
+        uwy = jy / r;
       }
 #pragma unroll
       for (int i = 1; i < 9; ++i) {
@@ -1003,37 +1001,62 @@ __global__ void __launch_bounds__(BX) flow_kernel(const FlowArgs a) {
       }
     }
 
-    // BGK by opposite pairs (i, j): sum s = f_i + f_j, difference d.  The
-    // equilibrium's even part depends on rho and the products of j = rho u,
-    // its odd part on j alone, so one reciprocal of rho serves all nine, and
-    //   f_i', f_j' = h +- e,  h = (1 - om)/2 s + om even, e = (1 - om)/2 d + om odd.
-    const T s1 = f[1] + f[3], d1 = f[1] - f[3], s2 = f[2] + f[4], d2 = f[2] - f[4];
-    const T s5 = f[5] + f[7], d5 = f[5] - f[7], s6 = f[6] + f[8], d6 = f[6] - f[8];
-    const T rho = f[0] + ((s1 + s2) + (s5 + s6));
-    const T jx = d1 + (d5 - d6), jy = d2 + (d5 + d6);
-    const T q = reciprocal(rho);
-    const T keep = pick<T>(a.keep, a.fkeep), kh = pick<T>(a.kh, a.fkh);
-    const T k1 = pick<T>(a.k1, a.fk1), k3 = pick<T>(a.k3, a.fk3);
-    // 4.5 k1 (jx jx, jy jy, jx jy) / rho and k1 rho
-    const T q1 = pick<T>(a.k45, a.fk45) * q;
-    const T vx = jx * q1, vy = jy * q1;
-    const T X = vx * jx, Y = vy * jy, Z = vx * jy;
-    const T Q = X + Y;
-    const T t = k1 * rho - T(1) / T(3) * Q;   // om even of f_1 less X
-    const T t5 = Q + t;                       // 4 om even of f_5 less 2 Z
-    const T bx = k3 * jx, by = k3 * jy;
-    S *__restrict__ o = dst + n;
-    o[0] = P::store(keep * f[0] + T(4) * t);
-    auto put = [&](int i, int j, T h, T e) {
-      o[(long long)i * plane] = P::store(h + e);
-      o[(long long)j * plane] = P::store(h - e);
-    };
-    put(1, 3, kh * s1 + (X + t), kh * d1 + bx);
-    put(2, 4, kh * s2 + (Y + t), kh * d2 + by);
-    put(5, 7, T(0.25) * (T(2) * Z + t5) + kh * s5, T(0.25) * (bx + by) + kh * d5);
-    put(6, 8, T(0.25) * (T(-2) * Z + t5) + kh * s6, T(0.25) * (by - bx) + kh * d6);
+    T ux, uy;
+    if constexpr (sizeof(T) == 8) {
+      // BGK by opposite pairs (i, j): sum s = f_i + f_j, difference d.  The
+      // equilibrium's even part depends on rho and the products of j = rho u,
+      // its odd part on j alone, so one reciprocal of rho serves all nine, and
+      //   f_i', f_j' = h +- e,  h = (1 - om)/2 s + om even, e = (1 - om)/2 d + om odd.
+      const T s1 = f[1] + f[3], d1 = f[1] - f[3], s2 = f[2] + f[4], d2 = f[2] - f[4];
+      const T s5 = f[5] + f[7], d5 = f[5] - f[7], s6 = f[6] + f[8], d6 = f[6] - f[8];
+      const T rho = f[0] + ((s1 + s2) + (s5 + s6));
+      const T jx = d1 + (d5 - d6), jy = d2 + (d5 + d6);
+      const T q = reciprocal(rho);
+      const T keep = a.keep, kh = a.kh;
+      const T k1 = a.k1, k3 = a.k3;
+      // 4.5 k1 (jx jx, jy jy, jx jy) / rho and k1 rho
+      const T q1 = a.k45 * q;
+      const T vx = jx * q1, vy = jy * q1;
+      const T X = vx * jx, Y = vy * jy, Z = vx * jy;
+      const T Q = X + Y;
+      const T t = k1 * rho - T(1) / T(3) * Q;   // om even of f_1 less X
+      const T t5 = Q + t;                       // 4 om even of f_5 less 2 Z
+      const T bx = k3 * jx, by = k3 * jy;
+      S *__restrict__ o = dst + n;
+      o[0] = P::store(keep * f[0] + T(4) * t);
+      auto put = [&](int i, int j, T h, T e) {
+        o[(long long)i * plane] = P::store(h + e);
+        o[(long long)j * plane] = P::store(h - e);
+      };
+      put(1, 3, kh * s1 + (X + t), kh * d1 + bx);
+      put(2, 4, kh * s2 + (Y + t), kh * d2 + by);
+      put(5, 7, T(0.25) * (T(2) * Z + t5) + kh * s5, T(0.25) * (bx + by) + kh * d5);
+      put(6, 8, T(0.25) * (T(-2) * Z + t5) + kh * s6, T(0.25) * (by - bx) + kh * d6);
+      ux = jx * q;
+      uy = jy * q;
+    } else {
+      // single precision is bound by HBM, and its constants, rounded one by
+      // one, would let the pairs' density drift by 1e-8 a step
+      T rho = T(0), jx = T(0), jy = T(0);
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        rho += f[i];
+        jx += T(cx(i)) * f[i];
+        jy += T(cy(i)) * f[i];
+      }
+      ux = jx / rho;
+      uy = jy / rho;
+      const T uu = ux * ux + uy * uy;
+      const T om = a.fomega;
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        const T cu = T(cx(i)) * ux + T(cy(i)) * uy;
+        const T feq = Lattice<T>::w(i) * rho *
+                      (T(1) + T(3) * cu + T(4.5) * cu * cu - T(1.5) * uu);
+        dst[(long long)i * plane + n] = P::store(f[i] + om * (feq - f[i]));
+      }
+    }
     if (MODE == kFlowU || MODE == kFlowCheck) {
-      const T ux = jx * q, uy = jy * q;
       if (MODE == kFlowCheck) {
         acc[0][0] = absT(ux - U[n]) + absT(uy - U[plane + n]);
         acc[0][1] = absT(ux) + absT(uy);

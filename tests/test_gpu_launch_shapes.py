@@ -90,3 +90,20 @@ def test_flow_step_shapes(shape):
     assert np.abs(got[0] - ux).max() < 1e-13
     assert np.abs(got[1] - uy).max() < 1e-13
     assert info["residual"] == pytest.approx(res, rel=1e-8)
+
+
+@pytest.mark.parametrize("shape", [(65, 24), (250, 620)])
+def test_flow_f32_keeps_its_density(shape):
+    """The FP32 flow against the oracle after 400 steps: each step rounds to
+    6e-8, with a systematic part below that (the weights as floats add up to
+    1 - 3e-8), so the velocities stay within 400 * 6e-8 * 2 of 0.05 and
+    relative; a density that drifts by another 1e-7 a step would not."""
+    nx, ny = shape
+    fib = _fibers(nx, ny)
+    solid, _, _ = oracle.raster(nx, ny, fib, 0.0, 0.0)
+    geom = lbm.Geometry(nx, ny, fib, 0.0, 0.0).upload()
+    u, _ = lbm.lbm_flow_solve(geom, 0.8, 0.05, 400, precision=lbm.LBM_F32)
+    _, ux, uy, _ = oracle.flow_run(solid, 0.8, 0.05, 400)
+    got = u.cpu().numpy()[:, :, :nx].astype(np.float64)
+    err = np.sqrt(np.sum((got[0] - ux) ** 2 + (got[1] - uy) ** 2))
+    assert err <= 400 * 6e-8 * 2 * np.sqrt(np.sum(ux ** 2 + uy ** 2))
