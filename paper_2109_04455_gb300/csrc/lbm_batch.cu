@@ -62,7 +62,7 @@ inline long long chunk_len(int prec, int tile) {
 // count in stepc[parity ^ 1] for the next launch.
 template <class P, int NS, int MODE, int TILE>
 __global__ void __launch_bounds__(StepThreads<P, MODE, TILE>::value,
-                                  !P::kDev ? 1 : MODE == kAdrCheck ? 1024 / TILE : 1536 / TILE)
+                                  !P::kDev ? (sizeof(typename P::T) == 8 ? 1024 / TILE : 1) : MODE == kAdrCheck ? 1024 / TILE : 1536 / TILE)
     batch_step_kernel(const AdrArgs *__restrict__ table, int parity,
                       const unsigned long long *__restrict__ work,
                       long long nwork, double *partials, unsigned *stepc) {
