@@ -45,8 +45,7 @@ __host__ __device__ inline unsigned long long chunk_item(int inst,
 // Threads of a step's block: one node each, or with half storage four (plain
 // step) or two (check step) of a tile's nodes.  With one node per thread the
 // half batch took as long as the FP32 one: 390 us per step of 16 lattices, 7.9
-// million nodes, against 273 us with four (and 168 registers: at 128 they
-// spill, 286 us).
+// million nodes, against 273 us with four.
 template <class P, int MODE, int TILE>
 struct StepThreads {
   static constexpr int value = !P::kDev ? TILE : MODE == kAdrCheck ? TILE / 2 : TILE / 4;
@@ -56,13 +55,20 @@ inline long long chunk_len(int prec, int tile) {
   return prec == LBM_F16DEV ? tile / 4 : tile;
 }
 
+// Nodes in flight per SM asked of the register allocator, by steps of 16
+// lattices of 7.9 million nodes (three species): FP64 1024 (64 registers, 1.55
+// ms; 256 took 1.92), FP32 768 (80, 343 us; 512 took 373 and 1024 355), half
+// 1536 on plain steps (168, 273 us; 2048 spills, 286) and 1024 on check steps.
+template <class P, int MODE>
+constexpr int kStepNodes = P::kDev ? (MODE == kAdrCheck ? 1024 : 1536)
+                                   : sizeof(typename P::T) == 8 ? 1024 : 768;
+
 // stepc[parity]: steps every active instance has done before this one (all
 // start together); the launch passes it to the per-node updates as
 // AdrArgs::step (the rounding seed of half storage) and leaves the next
 // count in stepc[parity ^ 1] for the next launch.
 template <class P, int NS, int MODE, int TILE>
-__global__ void __launch_bounds__(StepThreads<P, MODE, TILE>::value,
-                                  !P::kDev ? (sizeof(typename P::T) == 8 ? 1024 / TILE : 1) : MODE == kAdrCheck ? 1024 / TILE : 1536 / TILE)
+__global__ void __launch_bounds__(StepThreads<P, MODE, TILE>::value, kStepNodes<P, MODE> / TILE)
     batch_step_kernel(const AdrArgs *__restrict__ table, int parity,
                       const unsigned long long *__restrict__ work,
                       long long nwork, double *partials, unsigned *stepc) {
