@@ -94,6 +94,9 @@ struct Args {
   int periodic;      // box periodic in x and y: no inlet, outlet or walls
   int homogeneous;   // every particle reacts, wherever it is
   int plain;         // step length outside unit_step's range
+  int moves;         // step length above zero
+  double dnx, dny;   // nx, ny
+  double xout, ytop; // nx - 1/2, ny - 1/2
   double dt, len, delta;   // time step, diffusion step length, shell width
   double hk1, hk2;         // homogeneous rates (A -> B, B -> C)
   unsigned long long seed;
@@ -185,6 +188,24 @@ __device__ inline float centred_float(unsigned long long z) {
              static_cast<unsigned>(z >> 32) ^ 0x80000000u)) * 0x1.0p-31f;
 }
 
+// v to float by shifting its bits, rounded towards zero (a conversion is an
+// FP64 operation): within 2^-23 of v for 2^-126 <= |v| < 2^127, 0 for smaller
+// values, NaN for larger ones.
+__device__ inline float shift_to_float(double v) {
+  constexpr unsigned kBias = (1023u - 127u) << 20;
+  const unsigned hi = __double2hiint(v), lo = __double2loint(v);
+  const unsigned mag = hi & 0x7FFFFFFFu;
+  if (mag < kBias + (1u << 20)) return 0.0f;
+  if (mag >= kBias + (254u << 20)) return __uint_as_float(0x7FC00000u);
+  return __uint_as_float((hi & 0x80000000u) | ((mag - kBias) << 3) | (lo >> 29));
+}
+// a positive normal float to double
+__device__ inline double shift_to_double(float f) {
+  const unsigned e = __float_as_uint(f);
+  return __hiloint2double(static_cast<int>((e >> 3) + ((1023u - 127u) << 20)),
+                          static_cast<int>(e << 29));
+}
+
 // (len v1 / r, len v2 / r), r = sqrt(q), each operation correctly rounded.
 // The square root is Goldschmidt's iteration from a float estimate with
 // Markstein's final correction, the quotients Markstein's division by a
@@ -203,7 +224,7 @@ __device__ inline void unit_step(const Args &a, double v1, double v2, double q,
     sy = ddiv(n2, r);
     return;
   }
-  const double y0 = double(rsqrtf(__double2float_rn(q)));
+  const double y0 = shift_to_double(rsqrtf(shift_to_float(q)));
   double g = q * y0, h = 0.5 * y0;
   double e = fma(-g, h, 0.5);
   g = fma(g, e, g);
@@ -264,7 +285,8 @@ __device__ inline double wrap(double v, double lo, double span) {
 __device__ inline double shell_rate(const Args &a, int s, double px,
                                     double py, int first) {
   if (a.homogeneous) return s == 0 ? a.hk1 : (s == 1 ? a.hk2 : 0.0);
-  const float fx = __double2float_rn(px), fy = __double2float_rn(py);
+  if (first >= a.nfib) return 0.0;
+  const float fx = shift_to_float(px), fy = shift_to_float(py);
   for (int j = first; j < a.nfib; ++j) {
     if (!may_hold(a.near[j], fx, fy)) continue;
     const Fiber &f = a.fib[j];
@@ -321,8 +343,8 @@ __device__ inline void spawn(const Args &a, const Buf &out,
     if (keep) {
       const unsigned long long ps = particle_seed(a.seed, id);
       px = dadd(x0, dmul(wx, draw(ps, t, kSpawnDraw)));
-      py = dadd(-0.5, dmul(static_cast<double>(a.ny), draw(ps, t, kSpawnDraw + 1)));
-      const float fx = __double2float_rn(px), fy = __double2float_rn(py);
+      py = dadd(-0.5, dmul(a.dny, draw(ps, t, kSpawnDraw + 1)));
+      const float fx = shift_to_float(px), fy = shift_to_float(py);
       for (int k = 0; k < a.nfib && keep; ++k) {
         if (!may_hold(a.near[k], fx, fy)) continue;
         const Fiber &f = a.fib[k];
@@ -389,7 +411,7 @@ __global__ void __launch_bounds__(kThreads)
       // first candidate of the square inside the unit disc.  The float
       // squared radius is within 1e-6 of the double's, so only a candidate
       // near the rim or the centre needs the double.
-      if (a.len > 0.0) {
+      if (a.moves) {
         const unsigned long long c0 =
             ps + (static_cast<unsigned long long>(t) * kDraws + 1ull) * kGamma;
         unsigned long long z1 = 0, z2 = 0;
@@ -415,31 +437,30 @@ __global__ void __launch_bounds__(kThreads)
         py = dadd(py, sy);
       }
       // elastic reflections: walls y = -1/2, ny - 1/2 and the fibers
-      const double ytop = dsub(static_cast<double>(a.ny), 0.5);
       int first = a.nfib;   // the first fiber that may hold the particle
       for (int pass = 0; pass < kReflections; ++pass) {
         bool hit = false;
         if (a.periodic) {
-          px = wrap(px, -0.5, static_cast<double>(a.nx));
-          py = wrap(py, -0.5, static_cast<double>(a.ny));
+          px = wrap(px, -0.5, a.dnx);
+          py = wrap(py, -0.5, a.dny);
         } else {
           if (below(py, -0.5)) {
             py = dsub(-1.0, py);
             hit = true;
-          } else if (below(ytop, py)) {
-            py = dsub(dmul(2.0, ytop), py);
+          } else if (below(a.ytop, py)) {
+            py = dsub(dmul(2.0, a.ytop), py);
             hit = true;
           }
         }
-        float fx = __double2float_rn(px), fy = __double2float_rn(py);
+        float fx = shift_to_float(px), fy = shift_to_float(py);
         first = a.nfib;
         for (int k = 0; k < a.nfib; ++k) {
           if (!may_hold(a.near[k], fx, fy)) continue;
           first = min(first, k);
           if (reflect_fiber(a.fib[k], px, py)) {
             hit = true;
-            fx = __double2float_rn(px);
-            fy = __double2float_rn(py);
+            fx = shift_to_float(px);
+            fy = shift_to_float(py);
           }
         }
         if (!hit) break;
@@ -452,8 +473,7 @@ __global__ void __launch_bounds__(kThreads)
       }
       // inlet and outlet
       if (!a.periodic) {
-        const double xout = dsub(static_cast<double>(a.nx), 0.5);
-        if (!below(px, xout)) {
+        if (!below(px, a.xout)) {
           outflow = s;
           keep = false;
         } else if (below(px, -0.5)) {
@@ -708,9 +728,9 @@ extern "C" lbm_status lbm_rwpt_create(int32_t nx, int32_t ny,
       q.ny = std::sin(r[4]);
     }
     // A point held by the fiber has coordinates of at most |c| + reach, so
-    // rounding it and the centre to float and subtracting is off by less
-    // than 1.2e-7 (|c| + reach) in each coordinate; the slack is three times
-    // that.  (Infinities and NaN leave the fiber in the double test.)
+    // cutting it to float (2^-23), rounding the centre (2^-24) and subtracting
+    // is off by less than 2.4e-7 (|c| + reach) in each coordinate; the slack
+    // is more than that.  (Infinities and NaN leave the fiber in the double test.)
     const double reach = std::fabs(q.rp) + p->delta;
     const double d = reach + 1e-3 +
                      4e-7 * (std::fabs(q.cx) + std::fabs(q.cy) + 2.0 * reach);
@@ -756,6 +776,11 @@ extern "C" lbm_status lbm_rwpt_create(int32_t nx, int32_t ny,
   a.fib = d_fib;
   a.near = d_near;
   a.plain = a.len > 1e-100 && a.len < 1e100 ? 0 : 1;
+  a.moves = a.len > 0.0 ? 1 : 0;
+  a.dnx = nx;
+  a.dny = ny;
+  a.xout = a.dnx - 0.5;
+  a.ytop = a.dny - 0.5;
   r->seed_count = periodic ? 0 : static_cast<long long>(std::llround(p->density * ny));
   int dev = 0, sms = 1;
   cudaGetDevice(&dev);
