@@ -1035,8 +1035,14 @@ __global__ void __launch_bounds__(BX) flow_kernel(const FlowArgs a) {
           jx += T(cx(j)) * own[j];
           jy += T(cy(j)) * own[j];
         }
-        uwx = jx / r;
-        uwy = jy / r;
+        if constexpr (sizeof(T) == 8) {
+          const T q = reciprocal(r);
+          uwx = jx * q;
+          uwy = jy * q;
+        } else {
+          uwx = jx / r;
+          uwy = jy / r;
+        }
       }
 #pragma unroll
       for (int i = 1; i < 9; ++i) {
@@ -1133,15 +1139,19 @@ __global__ void __launch_bounds__(BX) flow_kernel(const FlowArgs a) {
 // launchers (one translation unit per precision instantiates them)
 // ---------------------------------------------------------------------------
 // Threads per block of a step (= nodes of a row segment, and entries of a
-// boundary chunk).  FP32 and FP64: 256, or 64 where 256 would leave SMs
-// without a block or cover a quarter more than the row (152 SMs with at
-// least four blocks of 256 each; a 200 x 100 lattice has 100 such blocks).
-// FP16 storage: 256-node segments throughout, which its kernels cover with
-// 64 (plain) and 128 (check) threads.
+// boundary chunk).  FP32 and FP64: 256 on large lattices, whose kernels bound
+// their registers to keep warps in flight, else 64, without that bound and
+// reaching every SM.  The line is where 256-thread blocks are sixteen per SM
+// for FP32 (1000 x 300, three species: 15.5 us per step with 256 threads and
+// 9.3 with 64; 700 x 400, two species: 7.7 and 6.5; 2048 x 512: 42 and 50),
+// four for FP64 (700 x 400, two species: 25 and 29 us; 200 x 100 has 100 such
+// blocks), and where they would cover a quarter more than the row.  FP16
+// storage: 256-node segments throughout, which its kernels cover with 64
+// (plain) and 128 (check) threads.
 inline int adr_block_x(int prec, int nx_pad, int ny) {
   if (prec == LBM_F16DEV) return kBlockX;
-  const long long seg = (nx_pad + 255) / 256;
-  return seg * ny < 4 * 152 || seg * 256 * 4 > 5LL * nx_pad ? 64 : 256;
+  const long long seg = (nx_pad + 255) / 256, few = prec == LBM_F64 ? 4 * 152 : 16 * 152;
+  return seg * ny < few || seg * 256 * 4 > 5LL * nx_pad ? 64 : 256;
 }
 // Grid of a step: nxb row segments per row, plus the columns of blocks that
 // take the boundary chunks of bthreads nodes.
