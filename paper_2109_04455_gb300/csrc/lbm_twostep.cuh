@@ -14,12 +14,13 @@ namespace lbm {
 //
 // The ring's fourth row lets one barrier per iteration do: what iteration
 // r + 1 overwrites was last read in iteration r - 1.  The loads of row r + 1
-// are issued before the second update of row r - 1, their lines prefetched
-// into L2 two rows earlier, its link word and velocity a row earlier.
+// are issued before that barrier and the second update of row r - 1, their
+// lines prefetched into L2 two rows earlier, its link word and velocity a row
+// earlier.
 //
 // A node's update costs as much as in the one-step kernel, and 16 warps per
 // SM (128 registers; 2 x 108 KB of ring) do not hide all of its latency, so
-// the step is not at HBM's rate any more: 1.70 ms per step of the 16384 x
+// the step is not at HBM's rate any more: 1.66 ms per step of the 16384 x
 // 4096 lattice of three species, against 2.31 ms for the one-step kernel at
 // 95% of the copy bandwidth.  Runs of at most 32 rows keep what all blocks
 // touch at a time within a few pages of every plane: with 128 rows a 4096 x
@@ -154,7 +155,6 @@ __global__ void __launch_bounds__(TwoStep<NS>::kBX, TwoStep<NS>::kBlocks)
         for (int i = 0; i < 9; ++i) o[(s * 9 + i) * BX] = g[s][i];
       }
     }
-    __syncthreads();
     {   // L2 prefetch, one segment per plane: whole 16-byte groups (nx_pad is
         // a multiple of 32, xs and xe of 4)
       const int yp = r + 1 + K::kPrefetch;
@@ -175,6 +175,7 @@ __global__ void __launch_bounds__(TwoStep<NS>::kBX, TwoStep<NS>::kBlocks)
     }
     const Row after = row(r + 2);
     if (next.lw != kSolidNode) load(r + 1, next.lw);
+    __syncthreads();
     // second step of row r - 1
     if (r > y0 && owned && prev.lw != kSolidNode) {
       const int y = wrap_y(r - 1);
