@@ -795,7 +795,7 @@ struct AdjLayout {
 static AdjLayout adj_layout(const lbm_geometry *g, const lbm_adr_params *p) {
   const size_t pl = static_cast<size_t>(plane_of(g));
   const size_t ns = static_cast<size_t>(p->nspecies);
-  const dim3 gr = adr_node_grid(g->nx_pad, g->ny);
+  const dim3 gr = adj_grid(p->precision, g->nx_pad, g->ny);
   AdjLayout l{};
   l.buf = align256(ns * 9 * pl * compute_bytes(p->precision));
   l.partials = align256(static_cast<size_t>(gr.x) * gr.y * 2 * 8);
@@ -880,7 +880,7 @@ extern "C" lbm_status lbm_adr_adjoint(lbm_adr_solver *s, int64_t max_steps,
   int32_t *fiber = reinterpret_cast<int32_t *>(b + 2 * l.buf + l.partials +
                                                l.scratch + l.result);
   const size_t pl = static_cast<size_t>(plane_of(g));
-  const dim3 gr = adr_node_grid(g->nx_pad, g->ny);
+  const dim3 gr = adj_grid(prec, g->nx_pad, g->ny);
   const long long rows = static_cast<long long>(gr.x) * gr.y;
 
   // forward outfluxes of the current state -> d eps / d N_s

@@ -1180,6 +1180,11 @@ inline dim3 adr_node_grid(int nx_pad, int ny) {
   return dim3(static_cast<unsigned>((nx_pad + kBlockX - 1) / kBlockX),
               static_cast<unsigned>(ny));
 }
+// of the adjoint: one node per thread
+inline dim3 adj_grid(int prec, int nx_pad, int ny) {
+  const int bx = adr_block_x(prec, nx_pad, ny);
+  return dim3(static_cast<unsigned>((nx_pad + bx - 1) / bx), static_cast<unsigned>(ny));
+}
 // boundary entries per chunk of a check step
 inline int adr_check_threads(int prec, int nx_pad, int ny) {
   return prec == LBM_F16DEV ? kPairThreads : adr_block_x(prec, nx_pad, ny);

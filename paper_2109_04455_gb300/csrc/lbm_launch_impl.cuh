@@ -80,15 +80,23 @@ cudaError_t launch_flow(int mode, const FlowArgs &a, cudaStream_t st, bool chain
                                             : launch_flow_bx<P, 256>(mode, a, st, chained);
 }
 
+template <class P, int NS, int BX>
+static cudaError_t launch_adjoint_bx(int mode, const AdjArgs &a, cudaStream_t st,
+                                     bool chained) {
+  using T = typename P::T;
+  const auto kernel = mode == kAdjCheck ? (a.periodic ? adj_kernel<T, NS, kAdjCheck, true, BX>
+                                                      : adj_kernel<T, NS, kAdjCheck, false, BX>)
+                                        : (a.periodic ? adj_kernel<T, NS, kAdjStep, true, BX>
+                                                      : adj_kernel<T, NS, kAdjStep, false, BX>);
+  return launch_chained(chained, kernel, adj_grid(sizeof(T) == 8 ? LBM_F64 : LBM_F32, a.nx_pad, a.ny),
+                        BX, st, a);
+}
 template <class P, int NS>
 static cudaError_t launch_adjoint_ns(int mode, const AdjArgs &a, cudaStream_t st,
                                      bool chained) {
-  using T = typename P::T;
-  const auto kernel = mode == kAdjCheck ? (a.periodic ? adj_kernel<T, NS, kAdjCheck, true>
-                                                      : adj_kernel<T, NS, kAdjCheck, false>)
-                                        : (a.periodic ? adj_kernel<T, NS, kAdjStep, true>
-                                                      : adj_kernel<T, NS, kAdjStep, false>);
-  return launch_chained(chained, kernel, adr_node_grid(a.nx_pad, a.ny), kBlockX, st, a);
+  const int bx = adr_block_x(sizeof(typename P::T) == 8 ? LBM_F64 : LBM_F32, a.nx_pad, a.ny);
+  return bx == 64 ? launch_adjoint_bx<P, NS, 64>(mode, a, st, chained)
+                  : launch_adjoint_bx<P, NS, 256>(mode, a, st, chained);
 }
 
 template <class P>
