@@ -200,10 +200,10 @@ class ClockSampler:
 # ---------------------------------------------------------------------------
 # roofline bookkeeping
 # ---------------------------------------------------------------------------
-# algorithmic double flops of one FP64 interior node update with the E table:
-# per species 8 additions for C and, per population, C E_i - g and
-# g + omega (...) as two FMAs (4 flops)
-FP64_FLOPS_PER_NODE = SPECIES * (8 + 9 * 4)
+# double flops of one FP64 interior node update with the E table: per species
+# and population, C E_i - g and g + omega (...) as two FMAs (4 flops); C itself
+# is summed on the integer units
+FP64_FLOPS_PER_NODE = SPECIES * 9 * 4
 
 
 def _peak_hbm():

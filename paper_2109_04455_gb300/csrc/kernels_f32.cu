@@ -6,7 +6,7 @@ namespace lbm {
 // fitting L2, and reading them half as often pays: 3000 x 1500 nodes of three
 // species took 161 us per step with one step per launch and 150 with two,
 // 4096 x 2048 306 and 262 (two species 216 and 170), 16384 x 4096 2310 and
-// 1700.  Below it does not (2048 x 1024: 79 and 89 us; 1000 x 900: 48 and
+// 1660.  Below it does not (2048 x 1024: 79 and 89 us; 1000 x 900: 48 and
 // 47), nor for one species (4096 x 2048: 130 and 127).  The kernel numbers
 // the populations of all species with 32 bits.
 bool two_step_pays(int prec, int ns, long long plane) {

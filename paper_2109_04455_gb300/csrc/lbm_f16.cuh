@@ -138,7 +138,7 @@ __device__ __forceinline__ __half2 round_pair(float lo, float hi, uint32_t h,
 }
 }  // namespace f16
 
-// FP16 bulk step, two nodes per thread: nodes (x0, x0 + 1), x0 even, of row
+// FP16 row segment, two nodes per thread: nodes (x0, x0 + 1), x0 even, of row
 // y.  Every plane is read as aligned half2 pairs.  A pull with c_ix = +1
 // takes the sources (x0 - 1, x0): the high half of the pair to the left and
 // the low half of the node's own pair; c_ix = -1 takes (x0 + 1, x0 + 2)
@@ -156,7 +156,6 @@ __device__ __forceinline__ __half2 round_pair(float lo, float hi, uint32_t h,
 // 5, 6, 7, 8), 15..17 the centre reference pairs of rows y - 1, y, y + 1,
 // 18..20 the left ones, 21..23 the right ones.
 constexpr int kPairThreads = kBlockX / 2;
-constexpr int kPairSlots = 24;
 __device__ __forceinline__ constexpr int side_slot(int i) {
   return i == 1 ? 9 : i == 3 ? 10 : i == 5 ? 11 : i == 6 ? 12 : i == 7 ? 13 : 14;
 }

@@ -6,13 +6,14 @@
 //   link words   [ny][nx_pad]  uint32, nibble j-1 = type of neighbour x+c_j
 //   rates        k_AB, k_BC [ny][nx_pad] double (read on catalytic links only)
 //   velocity     [2][ny][nx_pad]
-// One thread owns one node; a block covers kBlockX consecutive nodes of one
-// row, so every population plane is read and written with coalesced
-// accesses (the pull of a plane is a pure shift: each element of the source
-// plane is read exactly once per step).
+// One thread owns one node (two or four with half storage); a block covers
+// consecutive nodes of one row, so every population plane is read and written
+// with coalesced accesses (the pull of a plane is a pure shift: each element
+// of the source plane is read exactly once per step).
 //
-// The path is bandwidth bound (about 1 flop per byte in float), so there are
-// no tensor-core contractions here; what matters is bytes per node update.
+// There are no contractions here (about 1 flop per byte in float).  What
+// bounds a step: bytes in float and half on large lattices, the FP64 pipe in
+// double, and the latency of one launch on small lattices.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -223,18 +224,6 @@ __device__ __forceinline__ void check_add(T (&acc)[3 * NS], int s, T c, T prev) 
   acc[2 * s + 1] += absT(c);
   acc[2 * NS + s] = c < acc[2 * NS + s] ? c : acc[2 * NS + s];
 }
-
-// two-wide vector of a storage / compute type
-template <typename S> struct Vec2;
-template <> struct Vec2<double> { using type = double2; };
-template <> struct Vec2<float> { using type = float2; };
-template <> struct Vec2<__half> { using type = __half2; };
-
-template <typename S>
-__device__ __forceinline__ S zero_of() { return S(0); }
-template <>
-__device__ __forceinline__ __half zero_of<__half>() { return __float2half_rn(0.0f); }
-
 
 // Reference concentrations of the half path are themselves stored in half:
 // any reference works as long as the writer and every reader use the same
