@@ -465,7 +465,6 @@ extern "C" lbm_status lbm_adr_create(const lbm_geometry *g,
   a.nx_pad = g->nx_pad;
   a.abb_all = (p->flags & LBM_ADR_INLET_ABB_ALL) ? 1 : 0;
   a.nodewise = (p->flags & LBM_ADR_NODEWISE) ? 1 : 0;
-  a.periodic = g->periodic;
   for (int k = 0; k < 3; ++k) {
     const bool on = k < p->nspecies;
     a.omega[k] = on ? 1.0 / p->tau[k] : 0.0;

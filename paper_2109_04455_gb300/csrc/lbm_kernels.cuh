@@ -335,7 +335,6 @@ struct AdrArgs {
                             // beyond them takes boundary-node chunks
   int abb_all;              // anti-bounce-back inlet for every species
   int nodewise;             // every population of a reactive node reacts
-  int periodic;             // LBM_PERIODIC_X | LBM_PERIODIC_Y
   unsigned step;            // steps done before this one (rounding seed)
   int xp;                   // flux plane
   double omega[3];          // 1/tau per species

@@ -71,19 +71,19 @@ __global__ void __launch_bounds__(TwoStep<NS>::kBX, TwoStep<NS>::kBlocks)
   extern __shared__ float ring[];   // [4][NS * 9][BX]
   const int tid = threadIdx.x;
   const int x = blockIdx.x * K::kOwned - 1 + tid;
-  int xw = x < 0 || x >= a.nx ? -1 : x;
-  if (a.periodic & LBM_PERIODIC_X) xw = x < 0 ? a.nx - 1 : x == a.nx ? 0 : xw;
+  // Columns and rows beyond an edge are the other side's, whether the edge is
+  // periodic or not: only the link words say so, and they may be uploaded anew
+  // between launches.  Without periodic links no node reads them.
+  const int xw = x < 0 ? a.nx - 1 : x < a.nx ? x : x == a.nx ? 0 : -1;
   const bool owned = tid >= 1 && tid <= K::kOwned && x < a.nx;
-  const bool edge = !(a.periodic & LBM_PERIODIC_X) && (xw == 0 || xw == a.nx - 1);
+  const bool edge = xw == 0 || xw == a.nx - 1;
   const int y0 = blockIdx.y * rows, y1 = min(y0 + rows, a.ny);
   const unsigned plane = static_cast<unsigned>(a.plane), np = a.nx_pad;
   const float *__restrict__ src = static_cast<const float *>(a.src);
   float *__restrict__ dst = static_cast<float *>(a.dst);
   const float *__restrict__ U = static_cast<const float *>(a.u);
 
-  auto wrap_y = [&](int r) {
-    return !(a.periodic & LBM_PERIODIC_Y) ? r : r < 0 ? r + a.ny : r >= a.ny ? r - a.ny : r;
-  };
+  auto wrap_y = [&](int r) { return r < 0 ? r + a.ny : r >= a.ny ? r - a.ny : r; };
   struct Row {
     uint32_t lw;
     float ux, uy;
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(TwoStep<NS>::kBX, TwoStep<NS>::kBlocks)
   auto row = [&](int r) -> Row {
     const int y = wrap_y(r);
     Row k{kSolidNode, 0.0f, 0.0f};
-    if (xw >= 0 && r <= y1 && y >= 0 && y < a.ny) {
+    if (xw >= 0 && r <= y1) {
       const unsigned n = y * np + xw;
       k.lw = a.links[n];
       k.ux = U[n];

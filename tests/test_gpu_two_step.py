@@ -60,3 +60,26 @@ def test_two_steps_equal_single_steps(nx, ny, ns, flags, periodic):
     assert np.array_equal(a.state_save(), b.state_save())
     # and so is what a checked run reports
     assert a.run(6) == b.run(6)
+
+
+def test_two_steps_follow_a_new_upload():
+    """Edges made periodic and uploaded into the same workspace hold for a
+    solver that was created before, as they do for single steps."""
+    nx, ny = 2033, 2101
+    geom = lbm.Geometry(nx, ny, _fibers(nx, ny), 0.3, 0.2)
+    geom.upload()
+    u = torch.zeros((2, ny, geom.nx_pad), device="cuda")
+    u[:, :, :nx] = 0.03
+    prm = lbm.adr_params(2, [0.6, 0.8], c_in=(1.0, 0.3), precision=lbm.LBM_F32,
+                         neg_tol=-1.0)
+    a = lbm.ADRSolver(geom, prm, u).init()
+    b = lbm.ADRSolver(geom, prm, u).init()
+    ws = geom.ws.data_ptr()
+    for flags in (0, 3, 1, 2, 0):
+        geom.set_periodic(flags)
+        geom.upload()
+        assert geom.ws.data_ptr() == ws
+        a.run(4, check=False)
+        for _ in range(4):
+            b.run(1, check=False)
+        assert np.array_equal(a.state_save(), b.state_save())
