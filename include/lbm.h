@@ -339,7 +339,8 @@ size_t lbm_batch_ws_bytes(int32_t count, const lbm_geometry *const *geoms,
  * per lattice; check_every of params[0] for all, rounded up to even; a
  * lattice runs whole check intervals, so max_steps is rounded up to a
  * multiple of it; tol <= 0 runs exactly that many steps),
- * u[i] its device velocity.  ws holds every lattice's populations. */
+ * u[i] its device velocity (which may start at any value of a larger buffer:
+ * it need not be 256-byte aligned).  ws holds every lattice's populations. */
 lbm_status lbm_batch_create(int32_t count, const lbm_geometry *const *geoms,
                             const lbm_adr_params *params,
                             const void *const *u, void *ws, size_t ws_bytes,

@@ -118,9 +118,9 @@ __global__ void __launch_bounds__(StepThreads<P, MODE, TILE>::value, kStepNodes<
       const int x0 = static_cast<int>(item & 0xffffff) * TILE;
       if constexpr (P::kDev) {
         if constexpr (MODE == kAdrCheck)
-          pair_segment<NS, MODE, BX>(sa, y, x0, acc);
+          pair_segment<NS, MODE, BX, true>(sa, y, x0, acc);
         else
-          quad_segment<NS, BX>(sa, y, x0);
+          quad_segment<NS, BX, true>(sa, y, x0);
       } else {
         const int x = x0 + threadIdx.x;
         const long long n = (long long)y * sa.nx_pad + x;
@@ -521,6 +521,11 @@ extern "C" lbm_status lbm_batch_create(int32_t count,
     const int xp = params[i].x_plane < 0 ? geoms[i]->nx - 3 : params[i].x_plane;
     if (!u[i] || xp < 0 || xp >= geoms[i]->nx) {
       set_error("lbm_batch_create: missing velocity or flux plane outside");
+      return LBM_EINVAL;
+    }
+    // u[i] may be a view that starts at any value of a larger buffer
+    if (reinterpret_cast<uintptr_t>(u[i]) % comp_b(params[i].precision) != 0) {
+      set_error("lbm_batch_create: velocity not aligned to its values");
       return LBM_EINVAL;
     }
   }

@@ -1,7 +1,7 @@
 // FP16-deviation storage (populations stored as half of 2^14 (g - w_i R),
 // R the storing node's concentration, itself stored in half): the update of
-// interior nodes, four per thread (plain steps) and two (check steps).  Included by lbm_kernels.cuh after AdrArgs and the
-// lattice helpers.
+// interior nodes, four per thread (plain steps) and two (check steps).
+// Included by lbm_kernels.cuh after AdrArgs and the lattice helpers.
 #pragma once
 
 namespace lbm {
@@ -273,14 +273,29 @@ __device__ __forceinline__ void pair_update(const AdrArgs &a, int y, int x0,
   }
 }
 
+// Velocity components of two and of four consecutive nodes, by one wide load
+// where U, whose address mod 16 every such vector of it shares, allows that.
+// (Only a batch takes a U that starts at any float; a single lattice's solver
+// wants it aligned.)
+template <bool ANYU>
+__device__ __forceinline__ bool wide_u(const float *U, unsigned bytes) {
+  return !ANYU || (reinterpret_cast<uintptr_t>(U) & (bytes - 1u)) == 0;
+}
+__device__ __forceinline__ float2 load_u2(const float *p, bool wide) {
+  return wide ? *reinterpret_cast<const float2 *>(p) : make_float2(p[0], p[1]);
+}
+__device__ __forceinline__ float4 load_u4(const float *p, bool wide) {
+  return wide ? *reinterpret_cast<const float4 *>(p) : make_float4(p[0], p[1], p[2], p[3]);
+}
+
 // Nodes [xb, xb + 2 THREADS) of row y, two per thread, loaded species by
 // species: the block first sends the L2 prefetches for the segment
 // LBM_PREFETCH_ROWS_F16 rows below it.
-template <int NS, int MODE, int THREADS>
+template <int NS, int MODE, int THREADS, bool ANYU>
 __device__ __forceinline__ void pair_segment(const AdrArgs &a, int y, int xb,
                                              float (&acc)[2][3 * NS]) {
   if (LBM_PREFETCH_ROWS_F16 > 0)
-    prefetch_rows_f16<NS, THREADS>(a, y + LBM_PREFETCH_ROWS_F16, xb, 2 * THREADS);
+    prefetch_rows_f16<NS, THREADS, ANYU>(a, y + LBM_PREFETCH_ROWS_F16, xb, 2 * THREADS);
   const int x0 = xb + 2 * threadIdx.x;
   const long long n0 = (long long)y * a.nx_pad + x0;
   uint2 lw = make_uint2(kSolidNode, kSolidNode);
@@ -290,8 +305,8 @@ __device__ __forceinline__ void pair_segment(const AdrArgs &a, int y, int xb,
   wait_for_previous();
   const __half2 z2 = __float2half2_rn(0.0f);
   const float *__restrict__ U = static_cast<const float *>(a.u);
-  const float2 ux = *reinterpret_cast<const float2 *>(U + n0);
-  const float2 uy = *reinterpret_cast<const float2 *>(U + a.plane + n0);
+  const bool wide = wide_u<ANYU>(U, sizeof(float2));
+  const float2 ux = load_u2(U + n0, wide), uy = load_u2(U + a.plane + n0, wide);
   // each species' pairs are loaded as its arithmetic needs them (the stores
   // of one species keep the next one's loads behind them)
   pair_update<NS, MODE>(a, y, x0, in0, in1, ux, uy, [&](int s, int k) {
@@ -313,7 +328,7 @@ __global__ void __launch_bounds__(kPairThreads, 5)
   if (chunk >= 0)
     boundary_nodes<PrecF16Dev, NS, kAdrCheck, kPairThreads>(a, chunk, acc[0]);
   else
-    pair_segment<NS, kAdrCheck, kPairThreads>(a, blockIdx.y, blockIdx.x * kBlockX, acc);
+    pair_segment<NS, kAdrCheck, kPairThreads, false>(a, blockIdx.y, blockIdx.x * kBlockX, acc);
   wait_for_previous();   // the partial sums are one buffer
   const long long row = partial_row<kPairThreads>(a, chunk);
   if (row >= 0)
@@ -343,10 +358,10 @@ __global__ void __launch_bounds__(kPairThreads, 5)
 constexpr int kQuadThreads = kBlockX / 4;
 
 // Nodes [xb, xb + 4 THREADS) of row y, four per thread.
-template <int NS, int THREADS>
+template <int NS, int THREADS, bool ANYU>
 __device__ __forceinline__ void quad_segment(const AdrArgs &a, int y, int xb) {
   if (LBM_PREFETCH_ROWS_F16 > 0)
-    prefetch_rows_f16<NS, THREADS>(a, y + LBM_PREFETCH_ROWS_F16, xb, 4 * THREADS);
+    prefetch_rows_f16<NS, THREADS, ANYU>(a, y + LBM_PREFETCH_ROWS_F16, xb, 4 * THREADS);
   const int x0 = xb + 4 * threadIdx.x;
   if (x0 >= a.nx_pad) return;   // nx_pad is a multiple of 4: x0 + 3 < nx_pad
   const long long np = a.nx_pad, plane = a.plane;
@@ -358,8 +373,8 @@ __device__ __forceinline__ void quad_segment(const AdrArgs &a, int y, int xb) {
   const __half *src = static_cast<const __half *>(a.src);
   __half *__restrict__ dst = static_cast<__half *>(a.dst);
   const float *__restrict__ U = static_cast<const float *>(a.u);
-  const float4 ux = *reinterpret_cast<const float4 *>(U + n0);
-  const float4 uy = *reinterpret_cast<const float4 *>(U + plane + n0);
+  const bool wide = wide_u<ANYU>(U, sizeof(float4));
+  const float4 ux = load_u4(U + n0, wide), uy = load_u4(U + plane + n0, wide);
   float2 El[9], Eh[9];
   f16::eq2(make_float2(ux.x, ux.y), make_float2(uy.x, uy.y), El);
   f16::eq2(make_float2(ux.z, ux.w), make_float2(uy.z, uy.w), Eh);
@@ -485,7 +500,7 @@ __global__ void __launch_bounds__(kQuadThreads, LBM_QUAD_MIN_BLOCKS)
   static_assert(kQuadThreads % 32 == 0, "whole warps");
   const long long chunk = boundary_chunk(a);
   if (chunk < 0) {
-    quad_segment<NS, kQuadThreads>(a, blockIdx.y, blockIdx.x * kBlockX);
+    quad_segment<NS, kQuadThreads, false>(a, blockIdx.y, blockIdx.x * kBlockX);
   } else {
     float acc[3 * NS];
     boundary_nodes<PrecF16Dev, NS, kAdrStep, kQuadThreads>(a, chunk, acc);

@@ -663,8 +663,9 @@ __device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes) {
                :: "l"(p), "r"(bytes) : "memory");
 }
 // Nodes [xb, xb + width) of row yp, xb and width multiples of 32, by a block
-// of THREADS threads; rows outside the lattice are skipped.
-template <int NS, int THREADS>
+// of THREADS threads; rows outside the lattice are skipped.  ANYU: u may start
+// at any float (its segment is then taken from the 16-byte boundary before).
+template <int NS, int THREADS, bool ANYU>
 __device__ __forceinline__ void prefetch_rows_f16(const AdrArgs &a, int yp, int xb, int width) {
   constexpr int kPop = 9 * NS, kAll = kPop + NS + 3;
   if (yp >= a.ny) return;
@@ -682,7 +683,9 @@ __device__ __forceinline__ void prefetch_rows_f16(const AdrArgs &a, int yp, int 
     } else if (t < kPop + NS) {
       prefetch_l2(a.rsrc + (t - kPop) * plane + yp * np + xb, 2u * cnt);
     } else if (t < kPop + NS + 2) {
-      prefetch_l2(static_cast<const float *>(a.u) + (t - kPop - NS) * plane + yp * np + xb, 4u * cnt);
+      const float *p = static_cast<const float *>(a.u) + (t - kPop - NS) * plane + yp * np + xb;
+      if (ANYU) p = reinterpret_cast<const float *>(reinterpret_cast<uintptr_t>(p) & ~uintptr_t{15});
+      prefetch_l2(p, 4u * cnt);
     } else if (t < kAll) {
       prefetch_l2(a.links + yp * np + xb, 4u * cnt);
     }
