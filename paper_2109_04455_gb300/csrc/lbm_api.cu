@@ -213,14 +213,15 @@ extern "C" lbm_status lbm_flow_solve(const lbm_geometry *g,
   a.ny = g->ny;
   a.nx_pad = g->nx_pad;
   // k1 = w_1 / tau with its last five bits cleared (Veltkamp's split), so that
-  // 3 k1 and 4.5 k1 are exact, and 1 - 1/tau less what that and the rounding
-  // took from the weights: the step then conserves mass and momentum as the
-  // scheme with the rounded weights does.  (With each constant rounded by
-  // itself the density drifts by up to 1e-16 per step.)
-  const double om = 1.0 / p->tau, w1 = 1.0 / 9.0;
-  const double c = 33.0 * (om * w1);
-  a.k1 = c - (c - om * w1);
-  a.keep = (1.0 - om) + 9.0 * std::fma(om, w1, -a.k1);
+  // 3 k1, 4.5 k1 and 9 k1 are exact, and keep = 1 - 9 k1, exact too while tau is
+  // below 7: the step then conserves mass and momentum to the last rounding.
+  // (A keep that follows the rounded weights, as the plain formulas do, loses
+  // 5e-17 to 1e-16 of both per step: 9 w_1 is 1 - 6e-17.  That led the error:
+  // 1e-13 to 3e-13 of the velocities after 400 steps of a 333 x 151 lattice.)
+  const double om = 1.0 / p->tau;
+  const double c = 33.0 * (om * (1.0 / 9.0));
+  a.k1 = c - (c - om * (1.0 / 9.0));
+  a.keep = std::fma(-9.0, a.k1, 1.0);
   a.kh = 0.5 * a.keep;
   a.k3 = 3.0 * a.k1;
   a.k45 = 4.5 * a.k1;

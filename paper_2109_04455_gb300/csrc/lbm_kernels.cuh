@@ -954,8 +954,10 @@ __device__ __forceinline__ double reciprocal(double v) {
 // equilibria took about 140 double operations a node and 235 us per step of a
 // 2048 x 512 lattice; by opposite pairs it takes about 60 and 135 us.  (A 200 x
 // 100 lattice: 14.6 and 8.5 us, with 64-thread blocks that reach every SM.)
-// Against an 80-bit run of the same scheme both forms' velocities are off by
-// 1.1e-13 to 2.6e-13 after 400 steps, by the rounding of the weights.
+// With constants that conserve mass (lbm_flow_solve) its velocities are 2e-15
+// to 7e-15 off an 80-bit run of the same scheme after 400 steps, over tau 0.56
+// to 1.3 and six lattices; the former step's, whose rounded weights lose mass,
+// were 1.2e-13 to 2.8e-13 off.
 template <class P, int MODE, int BX>
 __global__ void __launch_bounds__(BX) flow_kernel(const FlowArgs a) {
   using S = typename P::S;
