@@ -125,13 +125,18 @@ __device__ inline double dmul(double a, double b) { return __dmul_rn(a, b); }
 __device__ inline double ddiv(double a, double b) { return __ddiv_rn(a, b); }
 
 __device__ inline long long bits(double v) { return __double_as_longlong(v); }
-// v < t, for a threshold t that is not zero, by integer comparison of the
-// bit patterns (a comparison in double is an FP64 operation); a NaN that
-// arithmetic made is greater than every number
-__device__ inline bool below(double v, double t) {
-  const long long a = bits(v), b = bits(t);
-  return (a ^ ((a >> 63) & 0x7FFFFFFFFFFFFFFFll)) <
-         (b ^ ((b >> 63) & 0x7FFFFFFFFFFFFFFFll));
+// v < t, for a threshold t that is not zero, by integer comparison of the bit
+// patterns (a comparison in double is an FP64 operation); a NaN counts as
+// beyond the infinity of its sign
+__device__ inline long long key(double v) {
+  return bits(v) ^ ((bits(v) >> 63) & 0x7FFFFFFFFFFFFFFFll);
+}
+__device__ inline bool below(double v, double t) { return key(v) < key(t); }
+// the same where a NaN matters, which a velocity field may hold, of either
+// sign: false for it (from -infinity up, by distance in one unsigned test)
+__device__ inline bool number_below(double v, double t) {
+  constexpr unsigned long long kLow = 0x800FFFFFFFFFFFFFull;   // key of -infinity
+  return key(v) - kLow < key(t) - kLow;
 }
 
 // floor(v) as a double and as an integer.  Adding 1.5 * 2^52 rounded down
@@ -471,9 +476,11 @@ __global__ void __launch_bounds__(kThreads)
         const double k = shell_rate(a, s, px, py, first);
         if (k > 0.0 && draw(ps, t, kReactDraw) < dmul(k, a.dt)) s += 1;
       }
-      // inlet and outlet
+      // inlet and outlet (a particle whose x is NaN leaves; a NaN of y costs
+      // further reflection passes above that move nothing, and turns x into
+      // NaN with the next step's advection)
       if (!a.periodic) {
-        if (!below(px, a.xout)) {
+        if (!number_below(px, a.xout)) {
           outflow = s;
           keep = false;
         } else if (below(px, -0.5)) {
