@@ -114,10 +114,11 @@ struct Buf {
 // Counters (device, unsigned long long): three particle counts in turn (of
 // the buffer read, of the buffer written, and one that the step clears for
 // the next), the outflow of each species since the last reset, the overflow
-// flag.  A count can pass the capacity when particles are dropped for lack
-// of room (the appends count them, the slots refuse them), so every reader
+// flag, and the blocks that have finished a step that may run out of room (zero
+// between steps).  A count can pass the capacity when particles are dropped for
+// lack of room (the appends count them, the slots refuse them), so every reader
 // takes min(count, capacity).
-enum { kCount = 0, kOut = 3, kOverflow = 6, kCounters = 8 };
+enum { kCount = 0, kOut = 3, kOverflow = 6, kDone = 7, kCounters = 8 };
 
 __device__ inline double dadd(double a, double b) { return __dadd_rn(a, b); }
 __device__ inline double dsub(double a, double b) { return __dsub_rn(a, b); }
@@ -378,18 +379,23 @@ __global__ void __launch_bounds__(kThreads)
 // One time step: the blocks below `movers` move every particle of `in`
 // (count in cnt[kin]) and append the survivors to `out` (count in cnt[kout],
 // zero on entry), the others append the m new entrance particles; the third
-// count, cnt[kclr], is cleared for the next step.
+// count, cnt[kclr], is cleared for the next step.  Particles in the box come
+// before new ones: where there might not be room for all, the entrance
+// particles wait until every survivor has its slot, and the last block to
+// finish appends them.
 __global__ void __launch_bounds__(kThreads)
     rwpt_step_kernel(const Args a, Buf in, Buf out, unsigned long long *cnt,
                      int kin, int kout, int kclr, long long cap, long long t,
                      unsigned long long id0, long long m, int movers) {
   if (blockIdx.x == 0 && threadIdx.x == 0) cnt[kclr] = 0ull;
+  const long long n = min(static_cast<long long>(cnt[kin]), cap);
+  const bool tight = n + m > cap;
   if (static_cast<int>(blockIdx.x) >= movers) {
-    spawn(a, out, cnt, kout, cap, t, id0, m, -0.5, 1.0, blockIdx.x - movers,
-          gridDim.x - movers);
+    if (!tight)
+      spawn(a, out, cnt, kout, cap, t, id0, m, -0.5, 1.0, blockIdx.x - movers,
+            gridDim.x - movers);
     return;
   }
-  const long long n = min(static_cast<long long>(cnt[kin]), cap);
   const long long stride = static_cast<long long>(movers) * kThreads;
   for (long long base = static_cast<long long>(blockIdx.x) * kThreads; base < n;
        base += stride) {
@@ -506,6 +512,17 @@ __global__ void __launch_bounds__(kThreads)
       out.s[slot] = s;
       out.id[slot] = id;
     }
+  }
+  if (tight) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      last = atomicAdd(cnt + kDone, 1ull) + 1ull == static_cast<unsigned long long>(movers);
+      if (last) cnt[kDone] = 0ull;
+    }
+    __syncthreads();
+    if (last) spawn(a, out, cnt, kout, cap, t, id0, m, -0.5, 1.0, 0, 1);
   }
 }
 
