@@ -453,7 +453,8 @@ lbm_status lbm_rwpt_reset_counts(lbm_rwpt *r, void *stream);
 
 /* Copy the particles, in the order of their ids, to host arrays of max_count
  * entries; *count receives their number (LBM_ENOMEM if it exceeds
- * max_count). */
+ * max_count).  They are those after every step enqueued so far, on any
+ * stream; calls on one system from several threads take turns. */
 lbm_status lbm_rwpt_particles(lbm_rwpt *r, void *stream, int64_t max_count,
                               int64_t *count, double *x, double *y,
                               int32_t *species, uint64_t *id);

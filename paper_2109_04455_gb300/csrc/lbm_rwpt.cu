@@ -37,6 +37,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -656,9 +657,24 @@ struct lbm_rwpt {
   long long seed_count = 0;    // entrance particles per step
   int grid = 0;
   bool started = false;
+  // The read-back sorts in the buffer that the next step writes, so it must
+  // not run beside a step or another read-back: the calls on a system take
+  // turns, and the read-back's stream waits for `done`, which follows the last
+  // work enqueued on whatever stream.
+  std::mutex turn;
+  cudaEvent_t done = nullptr;
 };
 
 namespace {
+
+// r->done follows what `st` holds now (nothing to record while a graph is
+// being captured: its work has not run)
+cudaError_t mark_done(lbm_rwpt *r, cudaStream_t st) {
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  const cudaError_t e = cudaStreamIsCapturing(st, &capturing);
+  if (e != cudaSuccess || capturing != cudaStreamCaptureStatusNone) return e;
+  return cudaEventRecord(r->done, st);
+}
 
 struct RwptLayout {
   size_t xy, id, s, fib, near, cnt, total;
@@ -815,6 +831,7 @@ extern "C" lbm_status lbm_rwpt_create(int32_t nx, int32_t ny,
     e = cudaMemcpy(d_fib, fib.data(), sizeof(Fiber) * fib.size(), cudaMemcpyHostToDevice);
   if (nfibers > 0 && e == cudaSuccess)
     e = cudaMemcpy(d_near, near.data(), sizeof(Near) * near.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&r->done, cudaEventDisableTiming);
   if (e != cudaSuccess) {
     delete r;
     return rfail("lbm_rwpt_create", e);
@@ -823,7 +840,11 @@ extern "C" lbm_status lbm_rwpt_create(int32_t nx, int32_t ny,
   return LBM_OK;
 }
 
-extern "C" void lbm_rwpt_destroy(lbm_rwpt *r) { delete r; }
+extern "C" void lbm_rwpt_destroy(lbm_rwpt *r) {
+  if (!r) return;
+  cudaEventDestroy(r->done);
+  delete r;
+}
 
 extern "C" lbm_status lbm_rwpt_init(lbm_rwpt *r, void *stream) {
   NvtxRange nvtx_range("lbm_rwpt_init");
@@ -832,6 +853,7 @@ extern "C" lbm_status lbm_rwpt_init(lbm_rwpt *r, void *stream) {
     return LBM_EINVAL;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  std::lock_guard<std::mutex> lock(r->turn);
   cudaError_t e = cudaMemsetAsync(r->cnt, 0, 8 * kCounters, st);
   r->cur = 0;
   r->count = 0;
@@ -847,6 +869,7 @@ extern "C" lbm_status lbm_rwpt_init(lbm_rwpt *r, void *stream) {
     e = cudaGetLastError();
   }
   r->next_id = static_cast<unsigned long long>(m);
+  if (e == cudaSuccess) e = mark_done(r, st);
   if (e != cudaSuccess) return rfail("lbm_rwpt_init", e);
   r->started = true;
   return LBM_OK;
@@ -860,6 +883,7 @@ extern "C" lbm_status lbm_rwpt_run(lbm_rwpt *r, int64_t nsteps, void *stream,
     return LBM_EINVAL;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  std::lock_guard<std::mutex> lock(r->turn);
   cudaError_t e = cudaSuccess;
   const long long entering = (r->seed_count + kThreads - 1) / kThreads;
   const int spawners = static_cast<int>(entering < r->grid ? entering : r->grid);
@@ -876,6 +900,7 @@ extern "C" lbm_status lbm_rwpt_run(lbm_rwpt *r, int64_t nsteps, void *stream,
     ++r->steps;
     ++r->window;
   }
+  if (e == cudaSuccess) e = mark_done(r, st);
   if (e != cudaSuccess) return rfail("lbm_rwpt_run", e);
   if (!info) return LBM_OK;
   unsigned long long h[kCounters] = {0};
@@ -908,8 +933,10 @@ extern "C" lbm_status lbm_rwpt_reset_counts(lbm_rwpt *r, void *stream) {
     set_error("lbm_rwpt_reset_counts: NULL argument");
     return LBM_EINVAL;
   }
-  cudaError_t e = cudaMemsetAsync(r->cnt + kOut, 0, 8 * 3,
-                                  static_cast<cudaStream_t>(stream));
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  std::lock_guard<std::mutex> lock(r->turn);
+  cudaError_t e = cudaMemsetAsync(r->cnt + kOut, 0, 8 * 3, st);
+  if (e == cudaSuccess) e = mark_done(r, st);
   if (e != cudaSuccess) return rfail("lbm_rwpt_reset_counts", e);
   r->window = 0;
   return LBM_OK;
@@ -951,9 +978,11 @@ extern "C" lbm_status lbm_rwpt_particles(lbm_rwpt *r, void *stream,
     return LBM_EINVAL;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  std::lock_guard<std::mutex> lock(r->turn);
   unsigned long long n = 0;
-  cudaError_t e = cudaMemcpyAsync(&n, r->cnt + kCount + r->count, 8,
-                                  cudaMemcpyDeviceToHost, st);
+  cudaError_t e = cudaStreamWaitEvent(st, r->done, 0);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(&n, r->cnt + kCount + r->count, 8, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return rfail("lbm_rwpt_particles", e);
   if (static_cast<long long>(n) > r->cap) n = static_cast<unsigned long long>(r->cap);
