@@ -257,9 +257,12 @@ def _ncu_traffic(precision: str, units_per_launch: int):
 
 
 def _steps_per_launch(geom, precision):
-    """Plain steps per launch (and per pass over memory): FP32 lattices of
-    2^22 nodes or more take two."""
-    return 2 if precision == "f32" and geom.nx_pad * geom.ny >= 1 << 22 else 1
+    """Plain steps per launch (and per pass over memory), as the library
+    takes them on this lattice."""
+    from paper_2109_04455_gb300 import lbm
+    prec = {"f64": lbm.LBM_F64, "f32": lbm.LBM_F32,
+            "f16dev": lbm.LBM_F16DEV}[precision]
+    return lbm.load().lbm_adr_steps_per_launch(prec, SPECIES, geom.nx, geom.ny)
 
 
 def _algorithmic_bytes(geom, w, precision):

@@ -256,6 +256,13 @@ lbm_status lbm_adr_init(lbm_adr_solver *s, void *stream);
 lbm_status lbm_adr_run(lbm_adr_solver *s, int64_t nsteps, void *stream,
                        lbm_solve_info *info);
 
+/* Unchecked time steps that lbm_adr_run takes per kernel launch on an nx x ny
+ * lattice: 2 where large FP32 lattices are updated twice per pass over memory,
+ * else 1 (0 for arguments no solver takes).  Host arithmetic only; for whoever
+ * counts launches or bytes, the state does not depend on it. */
+int32_t lbm_adr_steps_per_launch(int32_t precision, int32_t nspecies,
+                                 int32_t nx, int32_t ny);
+
 /* Copy C_s at the last checked step (device, [nspecies][ny][nx_pad], double
  * for LBM_F64 else float) to conc_out. */
 lbm_status lbm_adr_conc(lbm_adr_solver *s, void *conc_out, void *stream);

@@ -542,6 +542,14 @@ static cudaError_t adr_plain_steps(lbm_adr_solver *s, int64_t n, cudaStream_t st
   return e;
 }
 
+extern "C" int32_t lbm_adr_steps_per_launch(int32_t precision, int32_t nspecies,
+                                            int32_t nx, int32_t ny) {
+  if (precision < LBM_F64 || precision > LBM_F16DEV || nspecies < 1 || nspecies > 3 ||
+      nx < 4 || ny < 1 || ny > 65535)
+    return 0;
+  return two_step_pays(precision, nspecies, pad32(nx) * ny) ? 2 : 1;
+}
+
 extern "C" lbm_status lbm_adr_run(lbm_adr_solver *s, int64_t nsteps,
                                   void *stream, lbm_solve_info *info) {
   NvtxRange nvtx_range("lbm_adr_run");

@@ -117,6 +117,7 @@ _SIGS = {
     "lbm_adr_destroy": (None, [_P]),
     "lbm_adr_init": (ctypes.c_int, [_P, _P]),
     "lbm_adr_run": (ctypes.c_int, [_P, ctypes.c_int64, _P, _P]),
+    "lbm_adr_steps_per_launch": (ctypes.c_int32, [ctypes.c_int32] * 4),
     "lbm_adr_conc": (ctypes.c_int, [_P, _P, _P]),
     "lbm_adr_solve": (ctypes.c_int, [_P, _P, _P, _P, ctypes.c_size_t, _P, _P,
                                      _P]),
