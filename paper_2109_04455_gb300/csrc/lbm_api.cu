@@ -529,7 +529,7 @@ static cudaError_t adr_step(lbm_adr_solver *s, int mode, cudaStream_t st, bool c
 // n plain steps
 static cudaError_t adr_plain_steps(lbm_adr_solver *s, int64_t n, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
-  const bool two = two_step_pays(s->p.precision, s->p.nspecies, s->a.plane);
+  const bool two = two_step_pays(s->p.precision, s->p.nspecies, s->a.nx, s->a.ny);
   for (int64_t k = 0; k < n && e == cudaSuccess;) {
     if (two && n - k >= 2) {
       e = launch_adr_two_step(s->p.nspecies, adr_next(s, 2), st);
@@ -547,7 +547,7 @@ extern "C" int32_t lbm_adr_steps_per_launch(int32_t precision, int32_t nspecies,
   if (precision < LBM_F64 || precision > LBM_F16DEV || nspecies < 1 || nspecies > 3 ||
       nx < 4 || ny < 1 || ny > 65535)
     return 0;
-  return two_step_pays(precision, nspecies, pad32(nx) * ny) ? 2 : 1;
+  return two_step_pays(precision, nspecies, nx, ny) ? 2 : 1;
 }
 
 extern "C" lbm_status lbm_adr_run(lbm_adr_solver *s, int64_t nsteps,

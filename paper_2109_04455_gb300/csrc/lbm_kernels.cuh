@@ -1193,7 +1193,7 @@ template <class P>
 cudaError_t launch_adr(int ns, int mode, const AdrArgs &a, cudaStream_t st,
                        bool chained = false);
 // two plain steps in one launch (FP32), and whether they are worth it
-bool two_step_pays(int prec, int ns, long long plane);
+bool two_step_pays(int prec, int ns, int nx, int ny);
 cudaError_t launch_adr_two_step(int ns, const AdrArgs &a, cudaStream_t st);
 template <class P>
 cudaError_t launch_adr_flux(int ns, const void *g, const RefT *ref,

@@ -226,21 +226,24 @@ __global__ void __launch_bounds__(TwoStep<NS>::kBX, TwoStep<NS>::kBlocks)
   }
 }
 
-// Rows per run.  A run of `rows` rows takes rows + 2 iterations and about 1.5
-// more to start; the blocks of all runs share the SMs, with 0.7 of a wave
-// lost to the uneven end.
-inline int two_step_rows(int nx, int ny, int owned, int blocks) {
+// Rows per run, and what a launch then costs (in iterations of all the chip's
+// blocks).  A run of `rows` rows takes rows + 2 iterations and about 1.5 more
+// to start (a run of the whole height as long as rows + 1.5: it reads its edges
+// from L2); the blocks of all runs share the SMs, with 0.7 of a wave lost to the
+// uneven end.
+struct TwoStepPlan {
+  int rows;
+  double cost;
+};
+inline TwoStepPlan two_step_plan(int nx, int ny, int owned, int blocks) {
   const long long strips = (nx + owned - 1) / owned;
-  int best = 4;
-  double cost = -1.0;
+  TwoStepPlan best{4, -1.0};
   for (int rows = 4; rows <= 32; ++rows) {
     const long long n = strips * ((ny + rows - 1) / rows);
     const double c = (n / (152.0 * blocks) + 0.7) * (rows + 3.5);
-    if (cost < 0.0 || c <= cost) {
-      cost = c;
-      best = rows;
-    }
+    if (best.cost < 0.0 || c <= best.cost) best = {rows, c};
   }
+  if (ny <= best.rows) best.cost *= (best.rows + 1.5) / (best.rows + 3.5);
   return best;
 }
 

@@ -39,6 +39,20 @@ def test_arguments_no_solver_takes(steps):
         assert steps(*args) == 0
 
 
+@pytest.mark.parametrize("nx,ny,two", [
+    # whole strips of 254 columns, or lattices so large that a strip in part
+    # idle does not matter
+    (2032, 2100, 2), (4096, 1100, 2), (2048, 4096, 2), (1020, 16000, 2),
+    (140000, 32, 2), (1 << 20, 4, 2), (600, 14000, 2), (160, 27000, 2),
+    # strips much of which is idle: single steps are faster
+    (2048, 2048, 1), (1020, 4200, 1), (1280, 3300, 1), (510, 8300, 1),
+    (430, 10000, 1), (260, 16384, 1), (256, 16500, 1), (300, 14500, 1)])
+def test_strip_fill(steps, nx, ny, two):
+    assert (nx + 31) // 32 * 32 * ny >= 1 << 22
+    for ns in (2, 3):
+        assert steps(lbm.LBM_F32, ns, nx, ny) == two
+
+
 @pytest.mark.parametrize("precision", ["f64", "f32", "f16dev"])
 @pytest.mark.parametrize("nx,ny", [(2048, 512), (16384, 4096), (65536, 4096)])
 def test_benchmark_counts_what_the_library_does(steps, precision, nx, ny):
