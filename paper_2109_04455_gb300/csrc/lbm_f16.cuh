@@ -324,16 +324,14 @@ __global__ void __launch_bounds__(kPairThreads, 5)
   float acc[2][3 * NS];   // check-step values of node x0 and of node x0 + 1
 #pragma unroll
   for (int k = 0; k < 3 * NS; ++k) acc[0][k] = acc[1][k] = 0.0f;
-  const long long chunk = boundary_chunk(a);
-  if (chunk >= 0)
-    boundary_nodes<PrecF16Dev, NS, kAdrCheck, kPairThreads>(a, chunk, acc[0]);
+  const StepBlock k = step_block(a);
+  if (k.chunk >= 0)
+    boundary_nodes<PrecF16Dev, NS, kAdrCheck, kPairThreads>(a, k.chunk, acc[0]);
   else
-    pair_segment<NS, kAdrCheck, kPairThreads, false>(a, blockIdx.y, blockIdx.x * kBlockX, acc);
+    pair_segment<NS, kAdrCheck, kPairThreads, false>(a, k.y, k.xb * kBlockX, acc);
   wait_for_previous();   // the partial sums are one buffer
-  const long long row = partial_row<kPairThreads>(a, chunk);
-  if (row >= 0)
-    block_partials_store<2 * NS, NS, 2, kPairThreads, float>(
-        acc, a.partials + row * (3 * NS));
+  block_partials_store<2 * NS, NS, 2, kPairThreads, float>(
+      acc, a.partials + partial_row(a, k) * (3 * NS));
 }
 
 // FP16 plain step, four nodes per thread: nodes x0 .. x0 + 3 (x0 a multiple
@@ -498,12 +496,12 @@ template <int NS>
 __global__ void __launch_bounds__(kQuadThreads, LBM_QUAD_MIN_BLOCKS)
     adr_step_quad_kernel(const AdrArgs a) {
   static_assert(kQuadThreads % 32 == 0, "whole warps");
-  const long long chunk = boundary_chunk(a);
-  if (chunk < 0) {
-    quad_segment<NS, kQuadThreads, false>(a, blockIdx.y, blockIdx.x * kBlockX);
+  const StepBlock k = step_block(a);
+  if (k.chunk < 0) {
+    quad_segment<NS, kQuadThreads, false>(a, k.y, k.xb * kBlockX);
   } else {
     float acc[3 * NS];
-    boundary_nodes<PrecF16Dev, NS, kAdrStep, kQuadThreads>(a, chunk, acc);
+    boundary_nodes<PrecF16Dev, NS, kAdrStep, kQuadThreads>(a, k.chunk, acc);
   }
 }
 

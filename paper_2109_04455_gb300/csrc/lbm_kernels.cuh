@@ -19,6 +19,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <type_traits>
 
@@ -331,8 +332,11 @@ struct AdrArgs {
   long long nbnd;           // number of boundary nodes
   long long plane;          // ny * nx_pad
   int nx, ny, nx_pad;
-  int nxb;                  // row segments of a step's grid; blockIdx.x
-                            // beyond them takes boundary-node chunks
+  int nxb;                  // row segments per row of a step's grid
+  unsigned chunks;          // its boundary chunks, spread over the blocks at
+  unsigned share;           // this density, times 2^32 (step_block)
+  unsigned rowmul;          // division by nxb of an interior block's number
+  int rowshift;
   int abb_all;              // anti-bounce-back inlet for every species
   int nodewise;             // every population of a reactive node reacts
   unsigned step;            // steps done before this one (rounding seed)
@@ -692,18 +696,27 @@ __device__ __forceinline__ void prefetch_rows_f16(const AdrArgs &a, int yp, int 
   }
 }
 
-// Boundary-node chunk of a step's grid.  A step is one launch: the blocks of
-// blockIdx.x < a.nxb update the interior nodes (link word 0) of one row
-// segment each, and those beyond take chunks of BX entries of the
-// boundary-node list with every link rule in place (both read only the old
-// populations and write disjoint nodes).  The chunk is the block's number
-// among the latter, spread over the rows; -1 for an interior block.  Two
-// launches on two streams, forked and joined by events every step, cost a
-// 1000 x 300 lattice 34 us per step, almost all of it host time.
-__device__ __forceinline__ long long boundary_chunk(const AdrArgs &a) {
-  return static_cast<int>(blockIdx.x) < a.nxb
-             ? -1
-             : (long long)(blockIdx.x - a.nxb) * gridDim.y + blockIdx.y;
+// What a block of a step's grid works on.  A step is one launch: most blocks
+// update the interior nodes (link word 0) of one row segment each, in the order
+// of the rows, and the others chunks of BX entries of the boundary-node list
+// with every link rule in place (both read only the old populations and write
+// disjoint nodes).  Two launches on two streams, forked and joined by events
+// every step, cost a 1000 x 300 lattice 34 us per step, almost all of it host
+// time.  (With a column of blocks for the chunks beside the segments, mostly
+// empty blocks on high lattices and a chunk from elsewhere in the list on each
+// row, a step of 100 x 20000 FP32 took 167 us, 123 in this form, of 20000 x 50
+// half 40 and 30, and of 700 x 400 FP32 with thin fibers everywhere 15.3 and 12.2.)
+struct StepBlock {
+  long long chunk;   // of the boundary-node list, -1: a row segment
+  int xb, y;         // the segment
+};
+__device__ __forceinline__ StepBlock step_block(const AdrArgs &a) {
+  const unsigned b = blockIdx.x;
+  const unsigned before = min(__umulhi(b, a.share), a.chunks);
+  if (min(__umulhi(b + 1u, a.share), a.chunks) != before) return {before, 0, 0};
+  const unsigned i = b - before;
+  const unsigned y = a.nxb == 1 ? i : __umulhi(i, a.rowmul) >> a.rowshift;
+  return {-1, static_cast<int>(i - y * a.nxb), static_cast<int>(y)};
 }
 template <class P, int NS, int MODE, int BX>
 __device__ __forceinline__ void boundary_nodes(const AdrArgs &a, long long chunk,
@@ -713,12 +726,9 @@ __device__ __forceinline__ void boundary_nodes(const AdrArgs &a, long long chunk
   const BoundaryNode b = a.bnodes[t];
   adr_boundary_node<P, NS, MODE>(a, b.n, b.links, acc);
 }
-// check-step partial row of this block: interior blocks row by row, then the
-// boundary chunks that exist (-1 for a block with neither)
-template <int BX>
-__device__ __forceinline__ long long partial_row(const AdrArgs &a, long long chunk) {
-  if (chunk < 0) return (long long)blockIdx.y * a.nxb + blockIdx.x;
-  return chunk * BX < a.nbnd ? (long long)gridDim.y * a.nxb + chunk : -1;
+// check-step partial row of a block: the segments row by row, then the chunks
+__device__ __forceinline__ long long partial_row(const AdrArgs &a, const StepBlock &k) {
+  return k.chunk < 0 ? (long long)k.y * a.nxb + k.xb : (long long)a.ny * a.nxb + k.chunk;
 }
 
 }  // namespace lbm
@@ -828,20 +838,18 @@ __global__ void __launch_bounds__(BX, BX == 256 ? P::kMinBlocks : 1)
   T acc[1][3 * NS];
 #pragma unroll
   for (int k = 0; k < 3 * NS; ++k) acc[0][k] = T(0);
-  const long long chunk = boundary_chunk(a);
-  if (chunk >= 0) {
-    boundary_nodes<P, NS, MODE, BX>(a, chunk, acc[0]);
+  const StepBlock k = step_block(a);
+  if (k.chunk >= 0) {
+    boundary_nodes<P, NS, MODE, BX>(a, k.chunk, acc[0]);
   } else {
-    const int x = blockIdx.x * BX + threadIdx.x;
-    const long long n = (long long)blockIdx.y * a.nx_pad + x;
+    const int x = k.xb * BX + threadIdx.x;
+    const long long n = (long long)k.y * a.nx_pad + x;
     const uint32_t lw = (x < a.nx_pad) ? a.links[n] : kSolidNode;
     if (lw == 0u) adr_interior_node<P, NS, MODE, BX == 64>(a, n, acc[0]);
   }
   if constexpr (MODE == kAdrCheck) {
     wait_for_previous();   // the partial sums are one buffer
-    const long long row = partial_row<BX>(a, chunk);
-    if (row >= 0)
-      block_partials_store<2 * NS, NS, 1, BX, T>(acc, a.partials + row * (3 * NS));
+    block_partials_store<2 * NS, NS, 1, BX, T>(acc, a.partials + partial_row(a, k) * (3 * NS));
   }
 }
 
@@ -1146,20 +1154,45 @@ inline int adr_block_x(int prec, int nx_pad, int ny) {
   const long long seg = (nx_pad + 255) / 256, few = prec == LBM_F64 ? 4 * 152 : 16 * 152;
   return seg * ny < few || seg * 256 * 4 > 5LL * nx_pad ? 64 : 256;
 }
-// Grid of a step: nxb row segments per row, plus the columns of blocks that
-// take the boundary chunks of bthreads nodes.
+// Grid of a step: nxb row segments per row and the boundary chunks of bthreads
+// nodes, in one dimension (step_block).
 struct AdrGrid {
   int nxb;            // row segments per row
   long long chunks;   // boundary chunks
-  dim3 grid;
+  long long blocks() const { return static_cast<long long>(nxb) * ny + chunks; }
+  int ny;
 };
 inline AdrGrid adr_grid(int nx_pad, int ny, long long nbnd, int bx, int bthreads) {
-  AdrGrid g;
-  g.nxb = (nx_pad + bx - 1) / bx;
-  g.chunks = (nbnd + bthreads - 1) / bthreads;
-  g.grid = dim3(static_cast<unsigned>(g.nxb + (g.chunks + ny - 1) / ny),
-                static_cast<unsigned>(ny));
-  return g;
+  return {(nx_pad + bx - 1) / bx, (nbnd + bthreads - 1) / bthreads, ny};
+}
+// The grid's numbers for step_block.  Where the chunks go: every other block from
+// the start, so that none of them, which take longest, starts late (evenly over
+// the grid 1000 x 300 FP32, three species, took 11.7 us per step instead of
+// 9.3, 2048 x 512 FP64 121 instead of 113); from twelve waves of blocks evenly,
+// so that the latency of their scattered loads hides behind the segments'
+// streams and they run near the segments whose lines they share (the list goes
+// by rows too), up to two waves from the end unless there are so many that the
+// segments alone would not fill that (4096 x 2048 half, one species and thin
+// fibers everywhere: 209 us per step up to two waves, 192 to the end).
+//
+// share is rounded up, so that after `span` blocks all chunks have been passed
+// (step_block takes no more).  i / nxb for i < 2^31 is i ceil(2^(31 + s) / nxb) /
+// 2^(31 + s), s the bits of nxb - 1: the product is off by less than i 2^s <
+// 2^(31 + s).
+inline void set_grid(AdrArgs &a, const AdrGrid &g, int bx) {
+  const long long wave = 152 * (bx == 64 ? 8 : 4), blocks = g.blocks();
+  long long span = 2 * g.chunks + 1;
+  if (blocks >= 12 * wave)
+    span = 6 * g.chunks >= blocks ? blocks : std::max(span, blocks - 2 * wave);
+  span = std::min(span, blocks);
+  a.nxb = g.nxb;
+  a.chunks = static_cast<unsigned>(g.chunks);
+  a.share = static_cast<unsigned>(
+      ((static_cast<unsigned long long>(g.chunks) << 32) + span - 1) / span);
+  int s = 1;
+  while ((1ll << s) < g.nxb) ++s;
+  a.rowshift = s - 1;
+  a.rowmul = static_cast<unsigned>(((1ull << (31 + s)) + g.nxb - 1) / g.nxb);
 }
 inline int flow_block_x(int nx_pad, int ny) {
   return adr_block_x(LBM_F32, nx_pad, ny);
@@ -1186,7 +1219,7 @@ inline int adr_check_threads(int prec, int nx_pad, int ny) {
 inline long long adr_partial_rows(int prec, int nx_pad, int ny, long long nbnd) {
   const AdrGrid g = adr_grid(nx_pad, ny, nbnd, adr_block_x(prec, nx_pad, ny),
                              adr_check_threads(prec, nx_pad, ny));
-  return static_cast<long long>(g.nxb) * ny + g.chunks;
+  return g.blocks();
 }
 
 template <class P>
