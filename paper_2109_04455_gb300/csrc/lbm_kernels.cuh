@@ -828,11 +828,21 @@ __global__ void __launch_bounds__(kBlockX)
   }
 }
 
+// 256-thread blocks per SM that the step bounds its registers by.  FP32 with one
+// species has nine loads a thread in flight, so it needs more threads than
+// with three: 4096 x 2048 took 130 us per step at four blocks, 113 at six, 2048 x
+// 512 12.3 and 10.4.
+template <class P, int NS>
+constexpr int step_blocks() {
+  return sizeof(typename P::T) == 4 && NS == 1 ? 6 : P::kMinBlocks;
+}
 // One step (or check step), one node per thread.  On large lattices (BX =
 // 256) the interior update needs its warps in flight, so the registers that
-// the boundary update would like are bounded (P::kMinBlocks blocks per SM).
+// the boundary update would like are bounded: with three species its 27 values
+// and 16 rates spill (1192 bytes of stores per thread in double, 92 in float),
+// which only boundary nodes pay for.
 template <class P, int NS, int MODE, int BX>
-__global__ void __launch_bounds__(BX, BX == 256 ? P::kMinBlocks : 1)
+__global__ void __launch_bounds__(BX, BX == 256 ? step_blocks<P, NS>() : 1)
     adr_step_kernel(const AdrArgs a) {
   using T = typename P::T;
   T acc[1][3 * NS];
@@ -966,8 +976,9 @@ __device__ __forceinline__ double reciprocal(double v) {
 // to 7e-15 off an 80-bit run of the same scheme after 400 steps, over tau 0.56
 // to 1.3 and six lattices; the former step's, whose rounded weights lose mass,
 // were 1.2e-13 to 2.8e-13 off.
-template <class P, int MODE, int BX>
-__global__ void __launch_bounds__(BX) flow_kernel(const FlowArgs a) {
+// BLOCKS: per SM, to bound the registers by (see flow_blocks_per_sm).
+template <class P, int MODE, int BX, int BLOCKS>
+__global__ void __launch_bounds__(BX, BLOCKS) flow_kernel(const FlowArgs a) {
   using S = typename P::S;
   using T = typename P::T;
   const int x = blockIdx.x * BX + threadIdx.x;
@@ -1196,6 +1207,17 @@ inline void set_grid(AdrArgs &a, const AdrGrid &g, int bx) {
 }
 inline int flow_block_x(int nx_pad, int ny) {
   return adr_block_x(LBM_F32, nx_pad, ny);
+}
+// 256-thread blocks per SM that the flow step bounds its registers by (0: none).
+// FP32 lattices whose populations don't fit L2 need the eight that 32 registers
+// allow, though their boundary nodes spill a little: 4096 x 2048 108 us per step
+// without a bound, 100 with; 2048 x 700 19.2 and 18.8; but 2048 x 512 11.5 and
+// 12.1.
+inline int flow_blocks_per_sm(int prec, int nx_pad, int ny) {
+  return prec == LBM_F32 && flow_block_x(nx_pad, ny) == 256 &&
+                 static_cast<long long>(nx_pad) * ny >= 5ll << 18
+             ? 8
+             : 0;
 }
 inline dim3 flow_grid(int nx_pad, int ny) {
   const int bx = flow_block_x(nx_pad, ny);

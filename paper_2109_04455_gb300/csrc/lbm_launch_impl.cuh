@@ -64,20 +64,25 @@ cudaError_t launch_adr_flux(int ns, const void *g, const RefT *ref,
   return cudaGetLastError();
 }
 
-template <class P, int BX>
+template <class P, int BX, int BLOCKS>
 static cudaError_t launch_flow_bx(int mode, const FlowArgs &a, cudaStream_t st,
                                   bool chained) {
-  const auto kernel = mode == kFlowStep ? flow_kernel<P, kFlowStep, BX>
-                      : mode == kFlowU  ? flow_kernel<P, kFlowU, BX>
-                      : mode == kFlowCheck ? flow_kernel<P, kFlowCheck, BX>
-                                           : flow_kernel<P, kFlowInit, BX>;
+  const auto kernel = mode == kFlowStep ? flow_kernel<P, kFlowStep, BX, BLOCKS>
+                      : mode == kFlowU  ? flow_kernel<P, kFlowU, BX, BLOCKS>
+                      : mode == kFlowCheck ? flow_kernel<P, kFlowCheck, BX, BLOCKS>
+                                           : flow_kernel<P, kFlowInit, BX, BLOCKS>;
   return launch_chained(chained, kernel, flow_grid(a.nx_pad, a.ny), BX, st, a);
 }
 
 template <class P>
 cudaError_t launch_flow(int mode, const FlowArgs &a, cudaStream_t st, bool chained) {
-  return flow_block_x(a.nx_pad, a.ny) == 64 ? launch_flow_bx<P, 64>(mode, a, st, chained)
-                                            : launch_flow_bx<P, 256>(mode, a, st, chained);
+  constexpr int kPrec = sizeof(typename P::T) == 8 ? LBM_F64 : LBM_F32;
+  if (flow_block_x(a.nx_pad, a.ny) == 64) return launch_flow_bx<P, 64, 0>(mode, a, st, chained);
+  if constexpr (kPrec == LBM_F32) {
+    if (flow_blocks_per_sm(kPrec, a.nx_pad, a.ny) == 8)
+      return launch_flow_bx<P, 256, 8>(mode, a, st, chained);
+  }
+  return launch_flow_bx<P, 256, 0>(mode, a, st, chained);
 }
 
 template <class P, int NS, int BX>
