@@ -793,17 +793,19 @@ __device__ __forceinline__ void adr_interior_node(const AdrArgs &a, long long n,
 }
 
 // Initial state g* of every node: C_A = 1, the others 0, at equilibrium, with
-// the source of step 0 on catalytic links.
+// the source of step 0 on catalytic links.  Bound by its stores: registers for
+// 1024 threads per SM (512 in double), and the rates loaded once for all species.
 template <class P, int NS>
-__global__ void __launch_bounds__(kBlockX)
+__global__ void __launch_bounds__(kBlockX, sizeof(typename P::T) == 8 ? 2 : 4)
     adr_init_kernel(const AdrArgs a) {
   using T = typename P::T;
   const int x = blockIdx.x * kBlockX + threadIdx.x, y = blockIdx.y;
   const long long n = (long long)y * a.nx_pad + x;
   const uint32_t lw = (x < a.nx_pad) ? a.links[n] : kSolidNode;
   if (lw == kSolidNode) return;
-  T E[9], C[NS];
+  T E[9], C[NS], ka[9], kb[9];
   adr_eq<P>(a, n, E);
+  const bool cat = lw != 0u && link_rates(a, lw, x, y, ka, kb);
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
     T g[9];
@@ -813,16 +815,6 @@ __global__ void __launch_bounds__(kBlockX)
     C[s] = c;
 #pragma unroll
     for (int i = 0; i < 9; ++i) g[i] = relax(om, c, E[i], g[i]);
-    T ka[9], kb[9];
-    bool cat = false;
-#pragma unroll
-    for (int j = 1; j < 9; ++j) {
-      if (nib(lw, j) != kCat) continue;
-      const long long m = neighbour(x, y, j, a.nx, a.ny, a.nx_pad);
-      ka[j] = T(a.kab[m]);
-      kb[j] = T(a.kbc[m]);
-      cat = true;
-    }
     if (cat) add_source<NS>(a, s, lw, ka, kb, C, g);
     put_node<P>(a, s, n, g, c);
   }
