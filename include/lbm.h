@@ -20,6 +20,10 @@
  *  - `stream` is a cudaStream_t passed as void* (NULL = legacy default
  *    stream).  Work is enqueued on it; calls that report numbers
  *    (lbm_flow_solve, lbm_adr_run with info, lbm_adr_solve) synchronise it.
+ *    The steps of one call overlap at their edges: a step reads link words,
+ *    rates and velocity before the one before it has ended.  So while a call
+ *    enqueues its steps, no other thread puts work that writes those on the
+ *    same stream (before and after the call it may).
  *  - Lattice: nodes (x, y), 0 <= x < nx (flow direction), 0 <= y < ny.  Device
  *    fields are row-major [ny][nx_pad], x contiguous, nx_pad = nx rounded up
  *    to a multiple of 32; multi-component fields put the component first
