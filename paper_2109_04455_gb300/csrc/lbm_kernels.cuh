@@ -27,9 +27,12 @@
 
 namespace lbm {
 
-// Launch shape of the lattice kernels:
-//   LBM_BLOCK_X        threads per block = nodes of one row segment of the
-//                      flow, initial-state and adjoint kernels
+// SMs of the part, for the rules on launch shapes and waves of blocks (a host
+// without a GPU evaluates them too, for the workspace sizes).
+constexpr int kSMs = 152;
+// Threads per block of the initial-state and gradient kernels, and nodes of a
+// row segment of half storage.  (The flow, step and adjoint kernels take 64 or
+// 256 threads, see adr_block_x.)
 #ifndef LBM_BLOCK_X
 #define LBM_BLOCK_X 256
 #endif
@@ -144,9 +147,10 @@ inline cudaError_t launch_chained(bool chained, void (*kernel)(P...), dim3 grid,
 
 // ---------------------------------------------------------------------------
 // deterministic block sum of K values in the value type A, stored by threads
-// 0..K-1 (one component each) to dst[0..K): used in double for the outflux
-// and for the adjoint's convergence measure.  (The forward check steps use
-// block_partials_store below, which sums in double whatever the precision.)
+// 0..K-1 (one component each) to dst[0..K): used in double for the outflux, and
+// in the run's precision for the adjoint's convergence measure.  (The forward
+// check steps use block_partials_store below, which sums in double whatever
+// the precision.)
 // ---------------------------------------------------------------------------
 template <int K, typename A>
 __device__ __forceinline__ void block_sum_store(const A (&v)[K], double *dst) {
@@ -276,9 +280,12 @@ __device__ __forceinline__ float sum_rn(const float (&g)[9]) { return sum_in_ord
 // up to eight roundings one after the other (over random populations the
 // largest error was 5.4e-16 of the largest term, 2.0e-15 in order).  Terms too
 // small or too large for that (the largest below 2^-943 or from 2^1016,
-// infinite, NaN) are added in order.  2048 x 512, three species: 163 us per
-// step in order, 113 in integers (with the species' loads one by one, see
-// adr_interior_node).
+// infinite, NaN) are added in order.  That holds for one sum; after a run both
+// forms are equally far off, by the rounding of the weights (300 to 1600 steps
+// of six lattices, one to three species: 1.5e-14 to 9.7e-14 off an 80-bit run,
+// within 1% of each other).  2048 x 512, three species: 163 us per step in order,
+// 113 in integers and with the species' loads one by one (adr_interior_node),
+// which were not timed apart.
 __device__ __forceinline__ double sum_rn(const double (&g)[9]) {
   unsigned top = 0u;
 #pragma unroll
@@ -412,12 +419,12 @@ __global__ void __launch_bounds__(256)
 // C_B), so every source term is known when its species is collided, and only
 // one species' nine populations need to be live at a time.
 
-// Where the update of a boundary node reads the old populations: the global
-// planes.  at(i, j, t) is the place of population i of the neighbour x + c_j
-// (j = 0: the node itself) across a link of type t (kFluid or kPeriodic),
-// get(s, place) its value for species s.  (The two-step kernel has another.)
+// Where the update of a boundary node (x, y), plane index n, reads the old
+// populations: the global planes.  at(i, j, t) is the place of population i of
+// the neighbour x + c_j (j = 0: the node itself) across a link of type t (kFluid
+// or kPeriodic), get(s, place) its value for species s.
 template <class P>
-struct GlobalSource {
+struct OldState {
   using T = typename P::T;
   struct Place {
     long long plane, node;   // i * plane, node index
@@ -491,17 +498,13 @@ __device__ __forceinline__ void add_source(const AdrArgs &a, int s, uint32_t lw,
 // place, and all are issued before any arithmetic: the boundary nodes'
 // latency bounds the step of a small lattice (a 200 x 100 one took 23 us per
 // step with each load behind its link's branch, species after species).
-template <int NS, class Src, typename T>
-__device__ __forceinline__ void gather_node(const Src &src, uint32_t lw, T (&g)[NS][9]) {
-  if (lw == 0u) {
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      const auto from = src.at(i, opp(i), kFluid);
-#pragma unroll
-      for (int s = 0; s < NS; ++s) g[s][i] = src.get(s, from);
-    }
-    return;
-  }
+//
+// (The two-step kernel gathers from global planes and from its ring by code of
+// its own, and has edge_rules over masks; both forms must stay alike, which the
+// tests of equal bits hold them to.)
+template <int NS, class P, typename T>
+__device__ __forceinline__ void gather_node(const OldState<P> &src, uint32_t lw,
+                                            T (&g)[NS][9]) {
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
     const uint32_t t = i == 0 ? (uint32_t)kFluid : nib(lw, opp(i));
@@ -570,8 +573,8 @@ __device__ __forceinline__ bool link_rates(const AdrArgs &a, uint32_t lw, int x,
 // a.nodewise, on all nine populations with the mean rates of those links (ka,
 // kb, cat: link_rates).  put(s, g, c) stores the new populations of species s,
 // whose concentration is c.
-template <int NS, class Src, typename T, class Put>
-__device__ __forceinline__ void update_node(const AdrArgs &a, const Src &src,
+template <int NS, class P, typename T, class Put>
+__device__ __forceinline__ void update_node(const AdrArgs &a, const OldState<P> &src,
                                             uint32_t lw, bool cat, const T (&ka)[9],
                                             const T (&kb)[9], const T (&E)[9],
                                             T (&g)[NS][9], Put &&put) {
@@ -630,7 +633,7 @@ __device__ __forceinline__ void adr_boundary_node(const AdrArgs &a, long long n,
   using T = typename P::T;
   const int y = static_cast<int>(n / a.nx_pad);
   const int x = static_cast<int>(n - (long long)y * a.nx_pad);
-  const GlobalSource<P> src{a, n, x, y};
+  const OldState<P> src{a, n, x, y};
   T g[NS][9], E[9], ka[9], kb[9], prev[NS];
   adr_eq<P>(a, n, E);
   const bool cat = link_rates(a, lw, x, y, ka, kb);
@@ -962,7 +965,7 @@ __device__ __forceinline__ double reciprocal(double v) {
 // One flow step.  The double step is bound by this part's FP64 pipe (two
 // lanes per clock and SM; HBM is busy to a tenth).  Two divisions and nine
 // equilibria took about 140 double operations a node and 235 us per step of a
-// 2048 x 512 lattice; by opposite pairs it takes about 60 and 135 us.  (A 200 x
+// 2048 x 512 lattice; by opposite pairs it takes about 60 and 130 us.  (A 200 x
 // 100 lattice: 14.6 and 8.5 us, with 64-thread blocks that reach every SM.)
 // With constants that conserve mass (lbm_flow_solve) its velocities are 2e-15
 // to 7e-15 off an 80-bit run of the same scheme after 400 steps, over tau 0.56
@@ -1154,7 +1157,7 @@ __global__ void __launch_bounds__(BX, BLOCKS) flow_kernel(const FlowArgs a) {
 // (plain) and 128 (check) threads.
 inline int adr_block_x(int prec, int nx_pad, int ny) {
   if (prec == LBM_F16DEV) return kBlockX;
-  const long long seg = (nx_pad + 255) / 256, few = prec == LBM_F64 ? 4 * 152 : 16 * 152;
+  const long long seg = (nx_pad + 255) / 256, few = (prec == LBM_F64 ? 4 : 16) * kSMs;
   return seg * ny < few || seg * 256 * 4 > 5LL * nx_pad ? 64 : 256;
 }
 // Grid of a step: nxb row segments per row and the boundary chunks of bthreads
@@ -1183,7 +1186,7 @@ inline AdrGrid adr_grid(int nx_pad, int ny, long long nbnd, int bx, int bthreads
 // 2^(31 + s), s the bits of nxb - 1: the product is off by less than i 2^s <
 // 2^(31 + s).
 inline void set_grid(AdrArgs &a, const AdrGrid &g, int bx) {
-  const long long wave = 152 * (bx == 64 ? 8 : 4), blocks = g.blocks();
+  const long long wave = kSMs * (bx == 64 ? 8 : 4), blocks = g.blocks();
   long long span = 2 * g.chunks + 1;
   if (blocks >= 12 * wave)
     span = 6 * g.chunks >= blocks ? blocks : std::max(span, blocks - 2 * wave);

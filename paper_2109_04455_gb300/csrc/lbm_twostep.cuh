@@ -20,7 +20,7 @@ namespace lbm {
 //
 // A node's update costs as much as in the one-step kernel, and 16 warps per
 // SM (128 registers; 2 x 108 KB of ring) do not hide all of its latency, so
-// the step is not at HBM's rate any more: 1.66 ms per step of the 16384 x
+// the step is not at HBM's rate any more: 1.68 ms per step of the 16384 x
 // 4096 lattice of three species, against 2.31 ms for the one-step kernel at
 // 95% of the copy bandwidth.  Runs of at most 32 rows keep what all blocks
 // touch at a time within a few pages of every plane: with 128 rows a 4096 x
@@ -240,7 +240,7 @@ inline TwoStepPlan two_step_plan(int nx, int ny, int owned, int blocks) {
   TwoStepPlan best{4, -1.0};
   for (int rows = 4; rows <= 32; ++rows) {
     const long long n = strips * ((ny + rows - 1) / rows);
-    const double c = (n / (152.0 * blocks) + 0.7) * (rows + 3.5);
+    const double c = (n / (double(kSMs) * blocks) + 0.7) * (rows + 3.5);
     if (best.cost < 0.0 || c <= best.cost) best = {rows, c};
   }
   if (ny <= best.rows) best.cost *= (best.rows + 1.5) / (best.rows + 3.5);
