@@ -19,6 +19,8 @@ STEPS = 40
 # one node short of, at and past a segment; more chunks than rows (a chunk
 # column of its own per block); 256-thread segments (at least 608 of them,
 # padding below a quarter)
+# (250 x 620 alone takes the last, in the FP64 ADR step; the other 256-thread
+# forms and the other precisions are in test_gpu_launch_shapes_wide.py)
 SHAPES = [(63, 9), (64, 24), (65, 24), (129, 40), (24, 130), (250, 620),
           (513, 620)]
 

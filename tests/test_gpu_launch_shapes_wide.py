@@ -5,9 +5,9 @@ one), and 256-thread segments with a partial last one.
 256 threads are taken from four 256-node segments per SM for the FP64 ADR step
 (608 of them) and from sixteen for the flow and the FP32 step (2432), where
 they cover at most a quarter more than the row: 470 columns are two segments
-of a padded row of 480.  (250 x 620 is the only shape of 256-thread segments,
-FP64 ADR and one whole segment per row, in the list of the single-precision-
-free tests beside this one: 513 x 620 and all its flows take 64 threads.)
+of a padded row of 480.  (Of the shapes in test_gpu_launch_shapes.py 250 x 620
+alone takes 256-thread segments, one whole one per row, in the FP64 ADR step;
+513 x 620, whose padding is too wide, and all flows there take 64 threads.)
 Half storage covers 256-node segments at any size, four nodes per thread on
 plain steps and two on checked ones.
 
