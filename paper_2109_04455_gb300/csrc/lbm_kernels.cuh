@@ -1165,8 +1165,9 @@ inline int adr_block_x(int prec, int nx_pad, int ny) {
 struct AdrGrid {
   int nxb;            // row segments per row
   long long chunks;   // boundary chunks
-  long long blocks() const { return static_cast<long long>(nxb) * ny + chunks; }
   int ny;
+  long long blocks() const { return static_cast<long long>(nxb) * ny + chunks; }
+  dim3 dim() const { return dim3(static_cast<unsigned>(blocks())); }
 };
 inline AdrGrid adr_grid(int nx_pad, int ny, long long nbnd, int bx, int bthreads) {
   return {(nx_pad + bx - 1) / bx, (nbnd + bthreads - 1) / bthreads, ny};
@@ -1177,9 +1178,9 @@ inline AdrGrid adr_grid(int nx_pad, int ny, long long nbnd, int bx, int bthreads
 // 9.3, 2048 x 512 FP64 121 instead of 113); from twelve waves of blocks evenly,
 // so that the latency of their scattered loads hides behind the segments'
 // streams and they run near the segments whose lines they share (the list goes
-// by rows too), up to two waves from the end unless there are so many that the
-// segments alone would not fill that (4096 x 2048 half, one species and thin
-// fibers everywhere: 209 us per step up to two waves, 192 to the end).
+// by rows too), up to two waves from the end, or to the end where they are a
+// sixth of the blocks (4096 x 2048 half, one species and thin fibers everywhere:
+// 209 us per step up to two waves, 192 to the end).
 //
 // share is rounded up, so that after `span` blocks all chunks have been passed
 // (step_block takes no more).  i / nxb for i < 2^31 is i ceil(2^(31 + s) / nxb) /

@@ -14,9 +14,9 @@ static cudaError_t launch_step(AdrArgs a, cudaStream_t st, bool chained) {
     const AdrGrid g = adr_grid(a.nx_pad, a.ny, a.nbnd, kBlockX, kThreads);
     set_grid(a, g, kThreads);
     if constexpr (MODE == kAdrCheck)
-      return launch_chained(chained, adr_check_pair_kernel<NS>, dim3(static_cast<unsigned>(g.blocks())), kThreads, st, a);
+      return launch_chained(chained, adr_check_pair_kernel<NS>, g.dim(), kThreads, st, a);
     else
-      return launch_chained(chained, adr_step_quad_kernel<NS>, dim3(static_cast<unsigned>(g.blocks())), kThreads, st, a);
+      return launch_chained(chained, adr_step_quad_kernel<NS>, g.dim(), kThreads, st, a);
   } else {
     const int bx = adr_block_x(sizeof(typename P::S) == 8 ? LBM_F64 : LBM_F32,
                                a.nx_pad, a.ny);
@@ -24,7 +24,7 @@ static cudaError_t launch_step(AdrArgs a, cudaStream_t st, bool chained) {
     set_grid(a, g, bx);
     return launch_chained(chained, bx == 64 ? adr_step_kernel<P, NS, MODE, 64>
                                             : adr_step_kernel<P, NS, MODE, 256>,
-                          dim3(static_cast<unsigned>(g.blocks())), bx, st, a);
+                          g.dim(), bx, st, a);
   }
 }
 
