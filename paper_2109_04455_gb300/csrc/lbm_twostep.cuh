@@ -228,9 +228,8 @@ __global__ void __launch_bounds__(TwoStep<NS>::kBX, TwoStep<NS>::kBlocks)
 
 // Rows per run, and what a launch then costs (in iterations of all the chip's
 // blocks).  A run of `rows` rows takes rows + 2 iterations and about 1.5 more
-// to start (a run of the whole height as long as rows + 1.5: it reads its edges
-// from L2); the blocks of all runs share the SMs, with 0.7 of a wave lost to the
-// uneven end.
+// to start (on a lattice of one run or two rows + 1.5: its edges are in L2); the
+// blocks of all runs share the SMs, with 0.7 of a wave lost to the uneven end.
 struct TwoStepPlan {
   int rows;
   double cost;
@@ -243,7 +242,7 @@ inline TwoStepPlan two_step_plan(int nx, int ny, int owned, int blocks) {
     const double c = (n / (double(kSMs) * blocks) + 0.7) * (rows + 3.5);
     if (best.cost < 0.0 || c <= best.cost) best = {rows, c};
   }
-  if (ny <= best.rows) best.cost *= (best.rows + 1.5) / (best.rows + 3.5);
+  if (ny <= 2 * best.rows) best.cost *= (best.rows + 1.5) / (best.rows + 3.5);
   return best;
 }
 

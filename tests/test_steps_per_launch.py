@@ -39,18 +39,21 @@ def test_arguments_no_solver_takes(steps):
         assert steps(*args) == 0
 
 
-@pytest.mark.parametrize("nx,ny,two", [
-    # whole strips of 254 columns, or lattices so large that a strip in part
-    # idle does not matter
-    (2032, 2100, 2), (4096, 1100, 2), (2048, 4096, 2), (1020, 16000, 2),
-    (140000, 32, 2), (1 << 20, 4, 2), (600, 14000, 2), (160, 27000, 2),
+@pytest.mark.parametrize("nx,ny,two,three", [
+    # steps per launch with two and three species: whole strips of 254 columns,
+    # or lattices so large or flat that a strip in part idle does not matter
+    (4096, 2048, 2, 2), (16384, 1024, 2, 2), (140000, 32, 2, 2),
+    (1 << 20, 4, 2, 2), (2048, 8192, 2, 2),
+    # two species move less, and so gain less
+    (2032, 2100, 1, 2), (4096, 1100, 1, 2), (1020, 16000, 1, 2), (600, 14000, 1, 2),
     # strips much of which is idle: single steps are faster
-    (2048, 2048, 1), (1020, 4200, 1), (1280, 3300, 1), (510, 8300, 1),
-    (430, 10000, 1), (260, 16384, 1), (256, 16500, 1), (300, 14500, 1)])
-def test_strip_fill(steps, nx, ny, two):
+    (2048, 2048, 1, 1), (1020, 4200, 1, 1), (1280, 3300, 1, 1), (510, 8300, 1, 1),
+    (430, 10000, 1, 1), (260, 16384, 1, 1), (256, 16500, 1, 1), (300, 14500, 1, 1),
+    (160, 27000, 1, 1)])
+def test_strip_fill(steps, nx, ny, two, three):
     assert (nx + 31) // 32 * 32 * ny >= 1 << 22
-    for ns in (2, 3):
-        assert steps(lbm.LBM_F32, ns, nx, ny) == two
+    assert steps(lbm.LBM_F32, 2, nx, ny) == two
+    assert steps(lbm.LBM_F32, 3, nx, ny) == three
 
 
 @pytest.mark.parametrize("precision", ["f64", "f32", "f16dev"])
