@@ -505,6 +505,18 @@ __device__ __forceinline__ void add_source(const AdrArgs &a, int s, uint32_t lw,
 template <int NS, class P, typename T>
 __device__ __forceinline__ void gather_node(const OldState<P> &src, uint32_t lw,
                                             T (&g)[NS][9]) {
+  // Any fluid node.  (The boundary list holds none of link word 0, yet without
+  // this branch the allocator spills 28 bytes a thread more in the FP32 batch
+  // step, whose 16 lattices then take 69.5 ms instead of 68.3.)
+  if (lw == 0u) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const auto from = src.at(i, opp(i), kFluid);
+#pragma unroll
+      for (int s = 0; s < NS; ++s) g[s][i] = src.get(s, from);
+    }
+    return;
+  }
 #pragma unroll
   for (int i = 0; i < 9; ++i) {
     const uint32_t t = i == 0 ? (uint32_t)kFluid : nib(lw, opp(i));
